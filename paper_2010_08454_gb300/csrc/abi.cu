@@ -195,7 +195,6 @@ ppl_status ppl_infer_is_suffstat(const ppl_model* model, const ppl_data* data,
   PPL_TRY(check_ws(ws, ws_bytes, n_particles, data->len, &w));
   cudaStream_t s = (cudaStream_t)stream;
   PPL_TRY(reset_ws(w, false, s));
-  PPL_TRY(cuda_status(cudaMemsetAsync(out_dev, 0, sizeof(ppl_is_result), s)));
   // the statistics live in the scratch region, unused by likelihood weighting
   const int d_max = p.min_deg + p.n_deg - 1 + p.coef_offset;
   PPL_TRY(cuda_status(launch_suffstat(data->x, data->y, data->len, d_max, w.scratch(), s)));
@@ -485,7 +484,6 @@ ppl_status ppl_posterior_reduce(const ppl_model* model, const ppl_poly_particle*
   PPL_TRY(check_ws(ws, ws_bytes, n, 0, &w));
   cudaStream_t s = (cudaStream_t)stream;
   PPL_TRY(reset_ws(w, false, s));
-  PPL_TRY(cuda_status(cudaMemsetAsync(out_dev, 0, sizeof(ppl_is_result), s)));
   PPL_TRY(cuda_status(launch_posterior(p, particles, lw, n, w.hdr(), w.partials(), out_dev, s)));
   return PPL_OK;
 }

@@ -393,59 +393,336 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) stats_kernel(
 
 // ---------------------------------------------------------------------------
 // Posterior summary of an existing weighted population of records, one pass.
+//
+// HBM bounds it (36 B a particle), if a particle costs few instructions: each
+// lane keeps all four degrees' sums (S, S2 and, per coefficient, sum w d and
+// sum w d^2, d = c - ref) in registers for the whole pass, as f32x2 pairs, and
+// adds a particle to all four with its weight masked by degree: 28 paired
+// multiply-adds and no shuffle, barrier or branch.  The reference (ref, m_ref)
+// of a degree is shared by the warp's lanes, m_ref within kRebaseNats of the
+// best log-weight the warp has met, so that the weights stay in range and the
+// moments are taken around a point that carries weight.  When a better trace
+// turns up, the lanes move their sums to it exactly (A' = e (A + S g), B' =
+// e (B + g (2 A + S g)), g the shift of the reference, e the ratio of the
+// weights); a warp's maximum rises about ln(particles) times, so that path is
+// rare.  After 1, 2, 4, .. tiles the reference moves to the warp's weighted
+// mean so far: sums of w d then stay near 0 and round less (around a trace, the
+// mean of 2^22 unit normals came out 1.5 times further off).  Records and log-weights come through a ring of kPostStages cp.async
+// tiles per warp (no register held for a load in flight); nothing is shared
+// between warps until the end.
+// 2^24 records: 698 us with block-wide tiles of 1024 (56 masked sums reduced by
+// shuffles and ten barriers a tile), 146 us this way (4.1 TB/s; the copy rate would take 89).
 // ---------------------------------------------------------------------------
-constexpr int kPostPpt = 4;
+constexpr int kPostThreads = 512;  // one block per SM
+constexpr int kPostWarps = kPostThreads / 32;
+constexpr int kPostPer = 4;                 // particles of a lane per tile
+constexpr int kPostU = 2;                   // of these in registers at once
+constexpr int kPostTile = 32 * kPostPer;    // particles of a warp's tile
+constexpr int kPostStages = 3;              // tiles in flight per warp
+constexpr float kRebaseNats = 8.0f;
 
-__global__ void __launch_bounds__(kTpb) posterior_kernel(PolyParams p,
-                                                         const ppl_poly_particle* __restrict__ rec,
-                                                         const float* __restrict__ lwin,
-                                                         int64_t N, WsHeader* hdr,
-                                                         DegPartial* parts, ppl_is_result* res) {
-  __shared__ GroupScratch gs;
-  __shared__ DegPartial run[kMaxDegrees];
-  const int tid = threadIdx.x;
-  if (tid < kMaxDegrees) deg_empty(run[tid]);
+struct PostStage {
+  float4 rec[kPostTile * 2];
+  float lw[kPostTile];
+};
+// a warp's references: c[6], m_ref, the best log-weight met; and its index
+struct __align__(16) PostRef {
+  float v[kMaxDegrees][8];
+  int arg[kMaxDegrees];
+};
+constexpr size_t kPostSmem = (size_t)kPostWarps * kPostStages * sizeof(PostStage);
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kLeft>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(kLeft) : "memory");
+}
+
+// Issue one warp tile's copies (coalesced 16-byte words; past N zero-filled).
+__device__ __forceinline__ void post_fetch(PostStage* st, const ppl_poly_particle* rec,
+                                           const float* lwin, int64_t base, int64_t N, int lane) {
+  const float4* src = reinterpret_cast<const float4*>(rec + base) + lane;
+  const float* lsrc = lwin + base + lane;
+  if (base + kPostTile <= N) {  // a whole tile: one address, constant offsets
+#pragma unroll
+    for (int q = 0; q < 2 * kPostPer; ++q) cp_async16(&st->rec[q * 32 + lane], src + q * 32, 16);
+    if (lwin) {
+#pragma unroll
+      for (int q = 0; q < kPostPer; ++q) cp_async4(&st->lw[q * 32 + lane], lsrc + q * 32, 4);
+    }
+    return;
+  }
+  const int left = (int)(N - base);  // below kPostTile
+#pragma unroll
+  for (int q = 0; q < 2 * kPostPer; ++q) {
+    const bool in = q * 32 + lane < 2 * left;
+    cp_async16(&st->rec[q * 32 + lane], in ? src + q * 32 : reinterpret_cast<const float4*>(rec),
+               in ? 16 : 0);
+  }
+  if (lwin) {
+#pragma unroll
+    for (int q = 0; q < kPostPer; ++q) {
+      const bool in = q * 32 + lane < left;
+      cp_async4(&st->lw[q * 32 + lane], in ? lsrc + q * 32 : lwin, in ? 4 : 0);
+    }
+  }
+}
+
+// A lane's sums of one degree as f32x2 pairs.
+struct PostSums {
+  unsigned long long s12, A[kMaxCoef / 2], B[kMaxCoef / 2];
+};
+
+// Move a lane's sums to a reference g below the old one (g = old - new per
+// coefficient), rescaling the weights by ex.
+__device__ __forceinline__ void post_move(PostSums& a, const float (&g)[kMaxCoef], float ex) {
+  const float2 s = f2_unpack(a.s12);
+  const unsigned long long ee = f2_pack(ex, ex), ss = f2_pack(s.x, s.x);
+#pragma unroll
+  for (int j = 0; j < kMaxCoef / 2; ++j) {
+    const unsigned long long gg = f2_pack(g[2 * j], g[2 * j + 1]);
+    const unsigned long long A1 = f2_fma(ss, gg, a.A[j]);  // A + S g
+    a.B[j] = f2_mul(ee, f2_fma(gg, f2_add(a.A[j], A1), a.B[j]));
+    a.A[j] = f2_mul(ee, A1);
+  }
+  a.s12 = f2_pack(s.x * ex, s.y * ex * ex);
+}
+
+__global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
+    PolyParams p, const ppl_poly_particle* __restrict__ rec, const float* __restrict__ lwin,
+    int64_t N, WsHeader* hdr, DegPartial* parts, ppl_is_result* res) {
+  extern __shared__ __align__(16) unsigned char post_dyn[];
+  __shared__ PostRef refs[kPostWarps];
+  __shared__ DegPartial wparts[kPostWarps][kMaxDegrees];
+  __shared__ int any_nan;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  PostStage* ring = reinterpret_cast<PostStage*>(post_dyn) + warp * kPostStages;
+  PostRef& rf = refs[warp];
+  if (tid == 0) any_nan = 0;
+  if (lane < kMaxDegrees) {
+#pragma unroll
+    for (int j = 0; j < kMaxCoef; ++j) rf.v[lane][j] = 0.0f;
+    rf.v[lane][6] = rf.v[lane][7] = -INFINITY;
+    rf.arg[lane] = 0x7fffffff;
+  }
   __syncthreads();
-  const int64_t group = (int64_t)kTpb * kPostPpt;
-  const int64_t n_groups = (N + group - 1) / group;
+  PostSums a[kMaxDegrees];
+#pragma unroll
+  for (int k = 0; k < kMaxDegrees; ++k) {
+    a[k].s12 = 0ull;
+#pragma unroll
+    for (int j = 0; j < kMaxCoef / 2; ++j) a[k].A[j] = a[k].B[j] = 0ull;
+  }
   int nan = 0, bad = 0;
-  for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
-    float lw[kPostPpt], c[kPostPpt][kMaxCoef];
-    int d[kPostPpt], idx[kPostPpt];
+  const int64_t tiles = (N + kPostTile - 1) / kPostTile;
+  const int64_t step = (int64_t)gridDim.x * kPostWarps;
+  const int64_t t0 = (int64_t)warp * gridDim.x + blockIdx.x;
 #pragma unroll
-    for (int q = 0; q < kPostPpt; ++q) {
-      const int64_t i = g * group + (int64_t)q * kTpb + tid;
-      idx[q] = (int)i;
-      d[q] = -1;
-      lw[q] = -INFINITY;
+  for (int f = 0; f < kPostStages - 1; ++f) {
+    if (t0 + f * step < tiles) post_fetch(ring + f, rec, lwin, (t0 + f * step) * kPostTile, N, lane);
+    cp_async_commit();
+  }
+  int slot = 0;
+  unsigned done = 0;
+  for (int64_t t = t0; t < tiles; t += step) {
+    cp_async_wait<kPostStages - 2>();
+    __syncwarp();  // the tile's words were copied by all lanes; its predecessor's slot is read out
+    {
+      const int64_t tf = t + (kPostStages - 1) * step;
+      const int fs = slot == 0 ? kPostStages - 1 : slot - 1;
+      if (tf < tiles) post_fetch(ring + fs, rec, lwin, tf * kPostTile, N, lane);
+      cp_async_commit();
+    }
+    const PostStage& st = ring[slot];
+    slot = slot + 1 == kPostStages ? 0 : slot + 1;
+    const int left = (int)::min(N - t * kPostTile, (int64_t)kPostTile);
+    // kPostU particles at a time: their loads, exponentials and sums overlap
 #pragma unroll
-      for (int k = 0; k < kMaxCoef; ++k) c[q][k] = 0.0f;
-      if (i < N) {
-        const float4* src = reinterpret_cast<const float4*>(rec + i);
-        const float4 a = src[0], b = src[1];
-        c[q][0] = a.x;
-        c[q][1] = a.y;
-        c[q][2] = a.z;
-        c[q][3] = a.w;
-        c[q][4] = b.x;
-        c[q][5] = b.y;
-        const int dd = __float_as_int(b.z) - p.min_deg;
-        if ((unsigned)dd < (unsigned)p.n_deg) {
-          d[q] = dd;
-          lw[q] = lwin ? lwin[i] : 0.0f;
-        } else {
-          bad = 1;
+    for (int q0 = 0; q0 < kPostPer; q0 += kPostU) {
+      float4 r0[kPostU], r1[kPostU], f0[kPostU], f1[kPostU];
+      float lw[kPostU];
+      int d[kPostU];
+      bool rare = false;
+#pragma unroll
+      for (int u = 0; u < kPostU; ++u) {
+        const int e = (q0 + u) * 32 + lane;
+        r0[u] = st.rec[2 * e];
+        r1[u] = st.rec[2 * e + 1];
+        lw[u] = lwin ? st.lw[e] : 0.0f;
+        d[u] = __float_as_int(r1[u].z) - p.min_deg;
+        const bool ok = e < left && (unsigned)d[u] < (unsigned)p.n_deg;
+        d[u] = ok ? d[u] : -1;
+        const float4* rp = reinterpret_cast<const float4*>(rf.v[ok ? d[u] : 0]);
+        f0[u] = rp[0];
+        f1[u] = rp[1];
+        // no particle, NaN, or above the best of its degree so far
+        rare |= !ok || !(lw[u] <= f1[u].w);
+      }
+      if (__any_sync(0xffffffffu, rare)) {
+#pragma unroll 1
+        for (int u = 0; u < kPostU; ++u) {
+          // (selected by comparison: the arrays stay in registers)
+          float lu = lw[0];
+          int du = d[0];
+#pragma unroll
+          for (int v = 1; v < kPostU; ++v)
+            if (u == v) {
+              lu = lw[v];
+              du = d[v];
+            }
+          const int e = (q0 + u) * 32 + lane;
+          bad |= e < left && du < 0;
+          nan |= du >= 0 && lu != lu;
+          const bool up = du >= 0 && lu > rf.v[du >= 0 ? du : 0][7];
+          if (!__any_sync(0xffffffffu, up)) continue;
+          const float* cu = reinterpret_cast<const float*>(&st.rec[2 * (e - lane)]);
+#pragma unroll
+          for (int k = 0; k < kMaxDegrees; ++k) {
+            const bool mine = up && du == k;
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            const float mx = warp_max(mine ? lu : -INFINITY);
+            // lanes hold increasing indices: the first lane at the maximum is the lowest
+            const int src = __ffs(__ballot_sync(0xffffffffu, mine && lu == mx)) - 1;
+            const float m0 = rf.v[k][6];
+            if (!(mx <= m0 + kRebaseNats)) {
+              float g[kMaxCoef];
+#pragma unroll
+              for (int j = 0; j < kMaxCoef; ++j) g[j] = rf.v[k][j] - cu[8 * src + j];
+              post_move(a[k], g, m0 > -INFINITY ? expf(m0 - mx) : 0.0f);
+              __syncwarp();
+              if (lane < kMaxCoef) rf.v[k][lane] = cu[8 * src + lane];
+              if (lane == 0) rf.v[k][6] = mx;
+            }
+            if (lane == src) {
+              rf.v[k][7] = mx;
+              rf.arg[k] = (int)(t * kPostTile + e);
+            }
+            __syncwarp();
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kPostU; ++u) {
+          const float4* rp = reinterpret_cast<const float4*>(rf.v[d[u] >= 0 ? d[u] : 0]);
+          f0[u] = rp[0];
+          f1[u] = rp[1];
+          if (d[u] < 0) {  // no particle: a zero weight at the reference
+            lw[u] = -INFINITY;
+            r0[u] = f0[u];
+            r1[u] = f1[u];
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kPostU; ++u) {
+        // -inf and NaN log-weights carry nothing
+        const float w = lw[u] > -INFINITY ? expf(lw[u] - f1[u].z) : 0.0f;
+        const unsigned long long d2[kMaxCoef / 2] = {
+            f2_sub(f2_pack(r0[u].x, r0[u].y), f2_pack(f0[u].x, f0[u].y)),
+            f2_sub(f2_pack(r0[u].z, r0[u].w), f2_pack(f0[u].z, f0[u].w)),
+            f2_sub(f2_pack(r1[u].x, r1[u].y), f2_pack(f1[u].x, f1[u].y))};
+        unsigned long long q2[kMaxCoef / 2];
+#pragma unroll
+        for (int j = 0; j < kMaxCoef / 2; ++j) q2[j] = f2_mul(d2[j], d2[j]);
+        const unsigned long long one_w = f2_pack(1.0f, w);
+#pragma unroll
+        for (int k = 0; k < kMaxDegrees; ++k) {
+          const float wk = d[u] == k ? w : 0.0f;
+          const unsigned long long ww = f2_pack(wk, wk);
+          a[k].s12 = f2_fma(ww, one_w, a[k].s12);
+#pragma unroll
+          for (int j = 0; j < kMaxCoef / 2; ++j) {
+            a[k].A[j] = f2_fma(ww, d2[j], a[k].A[j]);
+            a[k].B[j] = f2_fma(ww, q2[j], a[k].B[j]);
+          }
         }
       }
     }
-    group_partial<kPostPpt>(lw, d, idx, c, gs);
-    if (tid < kMaxDegrees) deg_merge(run[tid], gs.out[tid]);
-    if (tid == 0) nan |= gs.nan;
+    // after 1, 2, 4, .. tiles: the references move to the means
+    ++done;
+    if ((done & (done - 1)) == 0) {
+#pragma unroll
+      for (int k = 0; k < kMaxDegrees; ++k) {
+        const float S = warp_sum(f2_unpack(a[k].s12).x);
+        if (!(S > 0.0f)) continue;  // the same for the whole warp
+        float g[kMaxCoef], c[kMaxCoef];
+#pragma unroll
+        for (int j = 0; j < kMaxCoef; ++j) {
+          const float2 v = f2_unpack(a[k].A[j / 2]);
+          const float r = rf.v[k][j];
+          c[j] = r + warp_sum(j & 1 ? v.y : v.x) / S;
+          g[j] = r - c[j];
+        }
+        post_move(a[k], g, 1.0f);
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+          for (int j = 0; j < kMaxCoef; ++j) rf.v[k][j] = c[j];
+        }
+      }
+      __syncwarp();
+    }
   }
-  __syncthreads();
-  if (tid < kMaxDegrees) parts[blockIdx.x * kMaxDegrees + tid] = run[tid];
-  if (tid == 0 && nan) record_status(&hdr->status, PPL_ENAN);
+  cp_async_wait<0>();
+  // the warp's partials: sums over its lanes, moved to the best trace's weight
+#pragma unroll
+  for (int k = 0; k < kMaxDegrees; ++k) {
+    const float2 s = f2_unpack(a[k].s12);
+    const float S = warp_sum(s.x), S2 = warp_sum(s.y);
+    float A[kMaxCoef], B[kMaxCoef];
+#pragma unroll
+    for (int j = 0; j < kMaxCoef / 2; ++j) {
+      const float2 av = f2_unpack(a[k].A[j]), bv = f2_unpack(a[k].B[j]);
+      A[2 * j] = warp_sum(av.x);
+      A[2 * j + 1] = warp_sum(av.y);
+      B[2 * j] = warp_sum(bv.x);
+      B[2 * j + 1] = warp_sum(bv.y);
+    }
+    if (lane == 0) {
+      DegPartial r;
+      deg_empty(r);
+      r.m = rf.v[k][7];
+      r.arg = rf.arg[k];
+      if (r.m > -INFINITY && S > 0.0f) {
+        const float ex = expf(rf.v[k][6] - r.m), inv = 1.0f / S;
+        r.S = S * ex;
+        r.S2 = S2 * ex * ex;
+#pragma unroll
+        for (int j = 0; j < kMaxCoef; ++j) {
+          const float sh = A[j] * inv;
+          r.mean[j] = rf.v[k][j] + sh;
+          r.M2[j] = fmaxf(fmaf(-sh, A[j], B[j]), 0.0f) * ex;
+        }
+      }
+      wparts[warp][k] = r;
+    }
+  }
+  if (__any_sync(0xffffffffu, nan) && lane == 0) any_nan = 1;
   if (bad) record_status(&hdr->status, PPL_EINVAL);
+  __syncthreads();
+  if (warp < kMaxDegrees) {
+    DegPartial r;
+    deg_empty(r);
+    if (lane < kPostWarps) r = wparts[lane][warp];
+#pragma unroll 1
+    for (int o = 1; o < kPostWarps; o <<= 1) {
+      const DegPartial other = deg_shfl_xor(r, o);
+      deg_merge(r, other);
+    }
+    if (lane == 0) parts[blockIdx.x * kMaxDegrees + warp] = r;
+  }
+  if (tid == 0 && any_nan) record_status(&hdr->status, PPL_ENAN);
   if (elect_last_block(&hdr->ticket[1]))
     finalize_partials(parts, gridDim.x, p.n_deg, p.min_deg, N, hdr, res);
 }
@@ -536,10 +813,17 @@ cudaError_t launch_stats(const float* lw, int64_t N, WsHeader* hdr, void* parts,
 cudaError_t launch_posterior(const PolyParams& p, const ppl_poly_particle* rec, const float* lw,
                              int64_t N, WsHeader* hdr, void* parts, ppl_is_result* res,
                              cudaStream_t s) {
-  const int64_t groups = (N + (int64_t)kTpb * kPostPpt - 1) / ((int64_t)kTpb * kPostPpt);
-  const int grid = (int)std::max<int64_t>(
-      1, std::min<int64_t>(groups, std::min<int64_t>((int64_t)num_sms() * 4, kMaxBlocks)));
-  posterior_kernel<<<grid, kTpb, 0, s>>>(p, rec, lw, N, hdr, (DegPartial*)parts, res);
+  int unused = 0;
+  const cudaError_t e = device_once((const void*)posterior_kernel, &unused, [](int*) {
+    return cudaFuncSetAttribute(posterior_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kPostSmem);
+  });
+  if (e != cudaSuccess) return e;
+  // one block per SM; fewer when a block's warps would not get a tile each
+  const int64_t blocks = (N + (int64_t)kPostTile * kPostWarps - 1) / ((int64_t)kPostTile * kPostWarps);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, num_sms()));
+  posterior_kernel<<<grid, kPostThreads, kPostSmem, s>>>(p, rec, lw, N, hdr, (DegPartial*)parts,
+                                                         res);
   return cudaGetLastError();
 }
 

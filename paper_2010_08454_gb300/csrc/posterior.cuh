@@ -1,7 +1,7 @@
 // One-pass posterior reduction of weighted line-fitting traces (§3.6.2 the
 // normalisation of the log-weights; Fig. 1 the returned coefficients).
 //
-// A group of traces (one block's particles of one instance) is reduced to a
+// A group of traces (one warp's or block's of one instance) is reduced to a
 // per-degree partial: the best log-weight m and its index, S = sum exp(lw - m),
 // S2 = sum exp(2 (lw - m)), and the weighted mean and second central moment
 // M2 = sum w (c - mean)^2 of every coefficient.  Within a group the moments are
@@ -86,243 +86,106 @@ __device__ __forceinline__ DegPartial ld_partial_cg(const DegPartial* src) {
   return o;
 }
 
-// Shared-memory scratch of group_partial.
-struct GroupScratch {
-  float wmax[kTpb / 32][kMaxDegrees];
-  int warg[kTpb / 32][kMaxDegrees];
-  float bmax[kMaxDegrees];
-  int barg[kMaxDegrees];
-  float ref[kMaxDegrees][kMaxCoef];
-  float sums[kTpb / 32][kMaxDegrees * (2 + 2 * kMaxCoef)];
-  DegPartial out[kMaxDegrees];
-  int nan;
-};
-
-// Reduce PPT traces per thread (lw, degree index d in [0, 4) or -1 when the
-// slot is empty, coefficients c) over the block into gs.out[0..3].  Every
-// thread of the block must call it.  Indices passed as `idx` are global trace
-// indices (lowest wins ties).
-template <int PPT>
-__device__ __forceinline__ void group_partial(const float (&lw)[PPT], const int (&d)[PPT],
-                                              const int (&idx)[PPT],
-                                              const float (&c)[PPT][kMaxCoef],
-                                              GroupScratch& gs) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // 1. best trace of every degree
-  float m[kMaxDegrees];
-  int a[kMaxDegrees];
-  int nan = 0;
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k) {
-    m[k] = -INFINITY;
-    a[k] = 0x7fffffff;
-  }
-#pragma unroll
-  for (int q = 0; q < PPT; ++q) {
-    nan |= (d[q] >= 0) & (lw[q] != lw[q]);
-#pragma unroll
-    for (int k = 0; k < kMaxDegrees; ++k)
-      if (d[q] == k && (lw[q] > m[k] || (lw[q] == m[k] && idx[q] < a[k]))) {
-        m[k] = lw[q];
-        a[k] = idx[q];
-      }
-  }
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, m[k], o);
-      const int oa = __shfl_xor_sync(0xffffffffu, a[k], o);
-      if (om > m[k] || (om == m[k] && oa < a[k])) {
-        m[k] = om;
-        a[k] = oa;
-      }
-    }
-    if (lane == 0) {
-      gs.wmax[warp][k] = m[k];
-      gs.warg[warp][k] = a[k];
-    }
-  }
-  nan = __any_sync(0xffffffffu, nan);
-  if (tid == 0) gs.nan = 0;
-  __syncthreads();
-  if (lane == 0 && nan) gs.nan = 1;
-  if (tid < kMaxDegrees) {
-    float bm = -INFINITY;
-    int ba = 0x7fffffff;
-    for (int w = 0; w < kTpb / 32; ++w)
-      if (gs.wmax[w][tid] > bm || (gs.wmax[w][tid] == bm && gs.warg[w][tid] < ba)) {
-        bm = gs.wmax[w][tid];
-        ba = gs.warg[w][tid];
-      }
-    gs.bmax[tid] = bm;
-    gs.barg[tid] = ba;
-  }
-  __syncthreads();
-  // 2. the best trace's coefficients become the shift of its degree
-#pragma unroll
-  for (int q = 0; q < PPT; ++q)
-    if (d[q] >= 0 && idx[q] == gs.barg[d[q]])
-#pragma unroll
-      for (int k = 0; k < kMaxCoef; ++k) gs.ref[d[q]][k] = c[q][k];
-  __syncthreads();
-  // 3. weighted sums around the shift
-  constexpr int V = 2 + 2 * kMaxCoef;
-  float acc[kMaxDegrees][V];
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k)
-#pragma unroll
-    for (int v = 0; v < V; ++v) acc[k][v] = 0.0f;
-#pragma unroll
-  for (int q = 0; q < PPT; ++q) {
-    if (d[q] < 0) continue;
-    const int dd = d[q];
-    const float w = (lw[q] > -INFINITY) ? expf(lw[q] - gs.bmax[dd]) : 0.0f;
-    float dc[kMaxCoef];
-#pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) dc[k] = c[q][k] - gs.ref[dd][k];
-#pragma unroll
-    for (int k = 0; k < kMaxDegrees; ++k) {
-      const float wk = (k == dd) ? w : 0.0f;
-      acc[k][0] += wk;
-      acc[k][1] = fmaf(wk, wk, acc[k][1]);
-#pragma unroll
-      for (int j = 0; j < kMaxCoef; ++j) {
-        const float t = wk * dc[j];
-        acc[k][2 + j] += t;
-        acc[k][2 + kMaxCoef + j] = fmaf(t, dc[j], acc[k][2 + kMaxCoef + j]);
-      }
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k)
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float x = warp_sum(acc[k][v]);
-      if (lane == 0) gs.sums[warp][k * V + v] = x;
-    }
-  __syncthreads();
-  // 4. one thread per degree forms the partial
-  if (tid < kMaxDegrees) {
-    const int k = tid;
-    float tot[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float x = 0.0f;
-      for (int w = 0; w < kTpb / 32; ++w) x += gs.sums[w][k * V + v];
-      tot[v] = x;
-    }
-    DegPartial& p = gs.out[k];
-    p.m = gs.bmax[k];
-    p.arg = gs.barg[k];
-    p.S = tot[0];
-    p.S2 = tot[1];
-    if (p.m == -INFINITY || !(tot[0] > 0.0f)) {
-      deg_empty(p);
-      p.m = gs.bmax[k];
-      p.arg = gs.barg[k];
-    } else {
-#pragma unroll
-      for (int j = 0; j < kMaxCoef; ++j) {
-        const float A = tot[2 + j] / tot[0];
-        p.mean[j] = gs.ref[k][j] + A;
-        p.M2[j] = fmaxf(tot[2 + kMaxCoef + j] - A * tot[2 + j], 0.0f);
-      }
-    }
-  }
-  __syncthreads();
-}
-
-// Summary of a population from its four per-degree partials, by the 32 lanes
-// of one warp (every lane calls it).  S and S2 are the per-degree sums around
-// each degree's maximum as double-floats.  No FP64 arithmetic but single
-// conversions and power-of-two scalings (GB300's FP64 pipe is narrow: a chain
-// of FP64 exp, log and divisions took about 7 us): the degree weights
-// e^(m_k - M) = 2^n_k w_k (exp_split, so a degree's mass keeps its relative
-// precision far below FP32's range), the masses w_k S_k and their total s in
-// double-float, log s by df_log, p(n) and the ESS as corrected FP32 quotients
-// scaled back by 2^n_k in FP64.  Lanes 0-23 take one (degree, coefficient)
-// variance each, lanes 0-5 one pooled mean each.
-__device__ __forceinline__ void write_summary_warp(const DegPartial (&p)[kMaxDegrees],
-                                                   const float2 (&S)[kMaxDegrees],
-                                                   const float2 (&S2)[kMaxDegrees], int n_deg,
+// Summary of a population from its four per-degree partials (in shared
+// memory), by the 32 lanes of one warp (every lane calls it).  S and S2 are
+// the per-degree sums around each degree's maximum as double-floats.  No FP64
+// arithmetic but single conversions and power-of-two scalings (GB300's FP64
+// pipe is narrow: a chain of FP64 exp, log and divisions took about 7 us): the
+// degree weights e^(m_k - M) = 2^n_k w_k (exp_split, so a degree's mass keeps
+// its relative precision far below FP32's range), the masses w_k S_k and their
+// total s in double-float, log s by df_log, p(n) and the ESS as corrected FP32
+// quotients scaled back by 2^n_k in FP64.  Lane k < 4 works out degree k, lanes
+// 0 and 1 the two logarithms, lanes 0-23 one (degree, coefficient) variance
+// each, lanes 0-5 one pooled mean each: the code runs once per launch, cold
+// in the instruction caches, so what bounds it is its length (one copy of
+// each function spread over lanes instead of four unrolled ones).
+__device__ __forceinline__ void write_summary_warp(const DegPartial* p, const float2* S,
+                                                   const float2* S2, int n_deg,
                                                    int min_deg, int64_t N, int32_t status,
                                                    ppl_is_result* res) {
   const int lane = threadIdx.x & 31;
-  float M = -INFINITY;
-  int32_t arg = -1;
-  for (int k = 0; k < n_deg; ++k)
-    if (p[k].m != -INFINITY && (p[k].m > M || (p[k].m == M && p[k].arg < arg))) {
-      M = p[k].m;
-      arg = p[k].arg;
+  const int k = lane & (kMaxDegrees - 1);  // (lanes 4.. repeat lanes 0-3 up to the shuffles)
+  const bool has = k < n_deg && p[k].m != -INFINITY;
+  const float mk = has ? p[k].m : -INFINITY;
+  const float2 Sk = S[k], S2k = S2[k];
+  float M = mk;
+  int32_t arg = has ? p[k].arg : 0x7fffffff;
+#pragma unroll
+  for (int o = 1; o < kMaxDegrees; o <<= 1) {
+    const float om = __shfl_xor_sync(0xffffffffu, M, o);
+    const int32_t oa = __shfl_xor_sync(0xffffffffu, arg, o);
+    if (om > M || (om == M && oa < arg)) {
+      M = om;
+      arg = oa;
     }
-  // degree k's mass 2^n[k] mw[k] and e^(2 (m_k - M)) S2_k; s, s2 their totals
+  }
+  if (M == -INFINITY) arg = -1;
+  // degree k's mass 2^n mw and e^(2 (m_k - M)) S2_k; s, s2 their totals
   // (terms below 2^-120 of the best degree's, which is at least 1, vanish
   // at double-float precision)
-  int n[kMaxDegrees];
-  float2 mw[kMaxDegrees];
-  float2 s = make_float2(0.0f, 0.0f), s2 = make_float2(0.0f, 0.0f);
+  int n = 0;
+  float2 mw = make_float2(0.0f, 0.0f), s = mw, s2 = mw;
+  if (has && Sk.x > 0.0f) {
+    // m_k - M = dh + dl exactly (TwoSum of two floats); e^dl = 1 + dl
+    const float dh = __fsub_rn(mk, M);
+    const float bb = __fsub_rn(dh, mk);
+    const float dl = __fsub_rn(__fsub_rn(mk, __fsub_rn(dh, bb)), __fadd_rn(M, bb));
+    const ExpSplit e = exp_split(dh);
+    const float2 w = df_add(make_float2(e.m, 0.0f), make_float2(__fmul_rn(e.m, dl), 0.0f));
+    n = e.n;
+    mw = df_mul(Sk, w);
+    if (e.n >= -120) s = df_mul(mw, exp2i(e.n));
+    if (e.n >= -60) s2 = df_mul(df_mul(df_mul(S2k, w), w), exp2i(2 * e.n));
+  }
 #pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k) {
-    n[k] = 0;
-    mw[k] = make_float2(0.0f, 0.0f);
-    if (k < n_deg && p[k].m != -INFINITY && S[k].x > 0.0f) {
-      // m_k - M = dh + dl exactly (TwoSum of two floats); e^dl = 1 + dl
-      const float dh = __fsub_rn(p[k].m, M);
-      const float bb = __fsub_rn(dh, p[k].m);
-      const float dl = __fsub_rn(__fsub_rn(p[k].m, __fsub_rn(dh, bb)), __fadd_rn(M, bb));
-      const ExpSplit e = exp_split(dh);
-      const float2 w = df_add(make_float2(e.m, 0.0f), make_float2(__fmul_rn(e.m, dl), 0.0f));
-      n[k] = e.n;
-      mw[k] = df_mul(S[k], w);
-      if (e.n >= -120) {
-        s = df_add(s, df_mul(mw[k], exp2i(e.n)));
-        if (e.n >= -60) s2 = df_add(s2, df_mul(df_mul(df_mul(S2[k], w), w), exp2i(2 * e.n)));
-      }
-    }
+  for (int o = 1; o < kMaxDegrees; o <<= 1) {
+    s = df_add(s, df_shfl_xor(s, o));
+    s2 = df_add(s2, df_shfl_xor(s2, o));
   }
   // p(n): the FP32 quotient mw / s scaled by 2^n (FP32 value for the pooled
   // means, FP64 for the output)
-  float pf[kMaxDegrees], pq[kMaxDegrees];
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k) {
-    pq[k] = (s.x > 0.0f && mw[k].x > 0.0f) ? df_div(mw[k], s) : 0.0f;
-    pf[k] = n[k] >= -120 ? __fmul_rn(pq[k], exp2i(n[k])) : 0.0f;
-  }
-  // lanes 0-23: (degree k, coefficient j) mean and variance
+  const float pq = (s.x > 0.0f && mw.x > 0.0f) ? df_div(mw, s) : 0.0f;
+  const float pf = n >= -120 ? __fmul_rn(pq, exp2i(n)) : 0.0f;
+  // lanes 0-23: (degree kk, coefficient j) mean and variance
   if (lane < kMaxDegrees * kMaxCoef) {
-    const int k = lane / kMaxCoef, j = lane % kMaxCoef;
-    const bool ok = k < n_deg && p[k].m != -INFINITY && S[k].x > 0.0f && p[k].S > 0.0f;
-    res->deg_mean[k][j] = ok ? (double)p[k].mean[j] : 0.0;
-    res->deg_var[k][j] = ok ? (double)__fdiv_rn(p[k].M2[j], p[k].S) : 0.0;
+    const int kk = lane / kMaxCoef, j = lane % kMaxCoef;
+    const bool ok = kk < n_deg && p[kk].m != -INFINITY && S[kk].x > 0.0f && p[kk].S > 0.0f;
+    res->deg_mean[kk][j] = ok ? (double)p[kk].mean[j] : 0.0;
+    res->deg_var[kk][j] = ok ? (double)__fdiv_rn(p[kk].M2[j], p[kk].S) : 0.0;
   }
-  // lanes 0-5: pooled coefficient means
-  if (lane < kMaxCoef) {
+  // pooled coefficient means (written by lanes 0-5) and the heaviest degree
+  {
+    const int j = lane < kMaxCoef ? lane : 0;
     float2 mc = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int k = 0; k < kMaxDegrees; ++k) {
-      const bool ok = k < n_deg && p[k].m != -INFINITY && S[k].x > 0.0f && p[k].S > 0.0f;
-      if (ok) mc = df_add(mc, df_prod(pf[k], p[k].mean[lane]));
+    float best_p = 0.0f;
+    int best = 0;
+#pragma unroll 1
+    for (int kk = 0; kk < kMaxDegrees; ++kk) {
+      const float pk = __shfl_sync(0xffffffffu, pf, kk);
+      if (pk > best_p) {
+        best_p = pk;
+        best = kk;
+      }
+      if (kk < n_deg && p[kk].m != -INFINITY && S[kk].x > 0.0f && p[kk].S > 0.0f)
+        mc = df_add(mc, df_prod(pk, p[kk].mean[j]));
     }
-    res->mean_c[lane] = df_to_double(mc);
+    if (lane < kMaxCoef) res->mean_c[lane] = df_to_double(mc);
+    if (lane == 0) res->map_deg = min_deg + best;
   }
   if (lane < kMaxDegrees) {
-    const int k = lane;
-    const bool has = k < n_deg && p[k].m != -INFINITY;
     // 2^n as an FP64 value (n >= -1022; smaller masses underflow to 0)
-    const double scale = n[k] >= -1022 ? __hiloint2double((n[k] + 1023) << 20, 0) : 0.0;
-    res->p_n[k] = (double)pq[k] * scale;
-    res->deg_max_lw[k] = has ? (double)p[k].m : -INFINITY;
+    const double scale = n >= -1022 ? __hiloint2double((n + 1023) << 20, 0) : 0.0;
+    res->p_n[k] = (double)pq * scale;
+    res->deg_max_lw[k] = has ? (double)mk : -INFINITY;
     res->deg_argmax[k] = has ? p[k].arg : -1;
   }
+  // lane 0: log s, lane 1: log N
+  const float2 lg = df_log(lane == 1 || !(s.x > 0.0f) ? df_from_i64(N) : s);
+  const float2 log_n = make_float2(__shfl_sync(0xffffffffu, lg.x, 1), __shfl_sync(0xffffffffu, lg.y, 1));
   if (lane == 0) {
-    int best = 0;
-    for (int k = 1; k < n_deg; ++k)
-      if (pf[k] > pf[best]) best = k;
     if (s.x > 0.0f) {
-      const float2 log_s = df_log(s), log_n = df_log(df_from_i64(N));
-      res->lse = (double)M + df_to_double(log_s);
-      res->log_z = (double)M + df_to_double(df_add(log_s, df_neg(log_n)));
+      res->lse = (double)M + df_to_double(lg);
+      res->log_z = (double)M + df_to_double(df_add(lg, df_neg(log_n)));
       res->ess = (double)df_div(df_mul(s, s), s2);
     } else {  // no finite weight
       res->lse = -INFINITY;
@@ -333,7 +196,6 @@ __device__ __forceinline__ void write_summary_warp(const DegPartial (&p)[kMaxDeg
     res->argmax = arg;
     res->n_particles = N;
     res->n_deg = n_deg;
-    res->map_deg = min_deg + best;
     res->status = status;
     res->pad = 0;  // every field is written: callers need not clear the result
   }
@@ -365,13 +227,16 @@ struct DegSums {
 
 // ---------------------------------------------------------------------------
 // Final merge of the per-block partials, by the last block: warp k merges
-// degree k's partials (FP32, a lane-strided chain then a shuffle tree); the
-// sums S, S2 are recombined in double-float around the merged maximum; warp
-// 0 writes the summary.
+// degree k's partials (merge_degree), warp 0 writes the summary.
 // ---------------------------------------------------------------------------
-// Warp `warp` (< kMaxDegrees) merges degree `warp` of G block partials: the
-// maximum, its index and the moments in FP32 (a lane-strided chain, then a
-// shuffle tree), then the sums S, S2 rescaled to the merged maximum.
+// Warp `warp` (< kMaxDegrees) merges degree `warp` of G block partials in two
+// passes over them: the maximum and its index first, then every partial's
+// sums rescaled to that maximum once and added (S, S2 and sum w (mean - ref)
+// in double-float, ref the mean of the partial that holds the maximum; second
+// moments in FP32), so the additions of a pass are independent and nothing
+// waits on a chain of pairwise merges, each with two exponentials and a
+// division.  (With sum w (mean - ref) in FP32 the mean of 2^22 unit normals
+// lost to the pairwise chain: 1.0e-6 against 6.4e-7 of its norm.)
 __device__ __forceinline__ void merge_degree(const DegPartial* parts, int G, int warp, int lane,
                                              DegPartial& a, DegSums& ds) {
   // This code runs once per launch, by one block, after the kernel's data
@@ -379,32 +244,83 @@ __device__ __forceinline__ void merge_degree(const DegPartial* parts, int G, int
   // stay rolled (fewer instruction fetches), and the next partial is loaded
   // while the current one is merged.
   deg_empty(a);
+  ds.zero();
+  const DegPartial* mine = parts + warp;
+  float M = -INFINITY;
+  int arg = 0x7fffffff, at = 0;
+#pragma unroll 4
+  for (int b = lane; b < G; b += 32) {
+    const float2 h = __ldcg(reinterpret_cast<const float2*>(mine + b * kMaxDegrees));
+    const int ha = __float_as_int(h.y);
+    if (h.x > M || (h.x == M && ha < arg)) {
+      M = h.x;
+      arg = ha;
+      at = b;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float om = __shfl_xor_sync(0xffffffffu, M, o);
+    const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+    const int ob = __shfl_xor_sync(0xffffffffu, at, o);
+    if (om > M || (om == M && oa < arg)) {
+      M = om;
+      arg = oa;
+      at = ob;
+    }
+  }
+  if (M == -INFINITY) return;  // the same for the whole warp
+  const DegPartial ref = ld_partial_cg(mine + at * kMaxDegrees);
+  float2 A[kMaxCoef];
+  float B[kMaxCoef];
+#pragma unroll
+  for (int k = 0; k < kMaxCoef; ++k) {
+    A[k] = make_float2(0.0f, 0.0f);
+    B[k] = 0.0f;
+  }
   DegPartial nxt;
-  if (lane < G) nxt = ld_partial_cg(parts + lane * kMaxDegrees + warp);
+  if (lane < G) nxt = ld_partial_cg(mine + lane * kMaxDegrees);
 #pragma unroll 1
   for (int b = lane; b < G; b += 32) {
     const DegPartial cur = nxt;
-    if (b + 32 < G) nxt = ld_partial_cg(parts + (b + 32) * kMaxDegrees + warp);
-    deg_merge(a, cur);
+    if (b + 32 < G) nxt = ld_partial_cg(mine + (b + 32) * kMaxDegrees);
+    if (cur.m == -INFINITY) continue;
+    const float e = expf(cur.m - M), w = cur.S * e;
+    ds.S = df_add(ds.S, df_prod(cur.S, e));
+    ds.S2 = df_add(ds.S2, df_mul(df_prod(cur.S2, e), e));
+#pragma unroll
+    for (int k = 0; k < kMaxCoef; ++k) {
+      const float d = cur.mean[k] - ref.mean[k];
+      A[k] = df_add(A[k], df_prod(w, d));
+      B[k] = fmaf(cur.M2[k], e, fmaf(w * d, d, B[k]));
+    }
   }
 #pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
-    const DegPartial other = deg_shfl_xor(a, o);
-    deg_merge(a, other);
-  }
-  ds.zero();
-  if (a.m != -INFINITY) {
-    float4 h = make_float4(-INFINITY, 0.0f, 0.0f, 0.0f);  // (m, arg, S, S2)
-    if (lane < G) h = __ldcg(reinterpret_cast<const float4*>(parts + lane * kMaxDegrees + warp));
-#pragma unroll 1
-    for (int b = lane; b < G; b += 32) {
-      const float4 cur = h;
-      if (b + 32 < G)
-        h = __ldcg(reinterpret_cast<const float4*>(parts + (b + 32) * kMaxDegrees + warp));
-      ds.add(cur.x, make_float2(cur.z, 0.0f), make_float2(cur.w, 0.0f), a.m);
+    ds.S = df_add(ds.S, df_shfl_xor(ds.S, o));
+    ds.S2 = df_add(ds.S2, df_shfl_xor(ds.S2, o));
+#pragma unroll
+    for (int k = 0; k < kMaxCoef; ++k) {
+      A[k] = df_add(A[k], df_shfl_xor(A[k], o));
+      B[k] += __shfl_xor_sync(0xffffffffu, B[k], o);
     }
   }
-  ds.warp_total();
+  a.m = M;
+  a.arg = arg;
+  a.S = ds.S.x;
+  a.S2 = ds.S2.x;
+  if (a.S > 0.0f) {
+    const float inv = __frcp_rn(a.S);
+#pragma unroll
+    for (int k = 0; k < kMaxCoef; ++k) {
+      // ref + A / S with the quotient's and the sum's remainders (they may cancel)
+      const float q = __fmul_rn(A[k].x, inv);
+      const float r = __fadd_rn(__fmaf_rn(-q, ds.S.x, A[k].x), __fmaf_rn(-q, ds.S.y, A[k].y));
+      const float2 mean = df_add(make_float2(ref.mean[k], 0.0f), make_float2(q, __fmul_rn(r, inv)));
+      a.mean[k] = mean.x;
+      a.M2[k] = fmaxf(fmaf(-q, A[k].x, B[k]), 0.0f);
+    }
+  }
 }
 
 __device__ __forceinline__ void finalize_partials(const DegPartial* parts, int G, int n_deg,

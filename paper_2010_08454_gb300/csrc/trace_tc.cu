@@ -141,19 +141,6 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Paired FP32 multiply and add (PTX f32x2), each half rounded as the scalar
-// instruction would round it.
-__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // One 32-byte record in a single 256-bit store (p 32-byte aligned).
 __device__ __forceinline__ void st_record_v8(void* p, const float (&c)[kMaxCoef], int n,
                                              uint32_t i) {
