@@ -501,7 +501,7 @@ ppl_status ppl_batched_status(const void* ws, ppl_stream stream);
  *    Step s (the counter, kept on the device) trains on pairs (s mod
  *    (n_pairs / batch)) batch .. + batch - 1 and writes its summed loss to
  *    loss_per_step[s]; nothing a step does depends on host values, so the
- *    enqueued work of one call (about 17 launches per step) can be captured
+ *    enqueued work of one call (four launches per step) can be captured
  *    once in a CUDA graph by the caller and replayed for every later block of
  *    steps.
  *  ppl_infer_is_learned: ppl_infer_is_batched with each instance's draws from

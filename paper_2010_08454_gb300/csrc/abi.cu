@@ -270,7 +270,7 @@ ppl_status ppl_gemm_bf16(const void* A, int64_t sam, int64_t sak, const void* B,
   PPL_TRY(reset_ws(w, false, s));
   return cuda_status(launch_umma_gemm(reinterpret_cast<const __nv_bfloat16*>(A), sam, sak,
                                       reinterpret_cast<const __nv_bfloat16*>(B), sbn, sbk, M, N,
-                                      K, nullptr, nullptr, 0, C, nullptr, &w.hdr()->status, s));
+                                      K, C, &w.hdr()->status, s));
 }
 
 ppl_status ppl_infer_is(const ppl_model* model, const ppl_data* data, int64_t n_particles,

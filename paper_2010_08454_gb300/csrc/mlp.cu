@@ -14,16 +14,11 @@
 #include <cuda_bf16.h>
 
 #include "kernels.h"
+#include "mlp.cuh"
 #include "poly.cuh"
 #include "rng.cuh"
 
 namespace ppl {
-
-constexpr int kIn = 64, kHid = 256, kOut = 48, kPts = 32;
-// parameter buffer layout (FP32): W1 | b1 | W2 | b2 | W3 | b3
-constexpr size_t kOffW1 = 0, kOffB1 = kOffW1 + kHid * kIn, kOffW2 = kOffB1 + kHid,
-                 kOffB2 = kOffW2 + kHid * kHid, kOffW3 = kOffB2 + kHid,
-                 kOffB3 = kOffW3 + kOut * kHid, kNumParams = kOffB3 + kOut;
 
 // ---------------------------------------------------------------------------
 // Features: one warp per data set; lane l holds point l; bitonic sort by
@@ -104,115 +99,24 @@ __global__ void __launch_bounds__(kTpb) forward_sim_kernel(PolyParams p, float o
   if (lane < kMaxCoef) c_out[(int64_t)warp * kMaxCoef + lane] = c[lane];
 }
 
-// ---------------------------------------------------------------------------
-// BF16 GEMM on the fifth-generation tensor cores (umma_gemm.cu):
-//   C[m, n] = sum_k A(m, k) B(n, k)  (+ bias[n]) (relu) (* [mask(m, n) > 0])
-// A(m, k) = A[m * sam + k * sak], B(n, k) = B[n * sbn + k * sbk]: any layout,
-// so the backward products read transposed operands in place.
-// ---------------------------------------------------------------------------
-struct GemmArgs {
-  const __nv_bfloat16* A;
-  int64_t sam, sak;
-  const __nv_bfloat16* B;
-  int64_t sbn, sbk;
-  int M, N, K;
-  const float* bias;
-  const __nv_bfloat16* mask;  // [M x N] row-major, multiply by (mask > 0)
-  int relu;
-  float* Cf;           // FP32 output [M x N] (ldc = N), optional
-  __nv_bfloat16* Cb;   // BF16 output [M x N], optional
-};
-
-// Split-K scratch of the network's products: the largest product (256 x
-// 256) in up to 16 K slices.
-constexpr size_t kSplitFloats = (size_t)16 * 256 * 256;
-
-static cudaError_t gemm(const GemmArgs& g, int32_t* status, cudaStream_t s, float* split = nullptr) {
-  return launch_umma_gemm(g.A, g.sam, g.sak, g.B, g.sbn, g.sbk, g.M, g.N, g.K, g.bias, g.mask,
-                          g.relu, g.Cf, g.Cb, status, s, split, split ? kSplitFloats : 0);
+// A parameter's gradient: the sum of its batch slices, in order.
+__device__ __forceinline__ float slice_sum(const float* __restrict__ partial, int S, int64_t i) {
+  float g = 0.0f;
+#pragma unroll 4
+  for (int z = 0; z < S; ++z) g += partial[(size_t)z * kNumParams + i];
+  return g;
 }
 
-// ---------------------------------------------------------------------------
-// Loss -log q per pair and its gradient with respect to the outputs (divided
-// by the batch size), one thread per pair; per-block loss sums.
-// ---------------------------------------------------------------------------
-struct ProposalShape {
-  int min_deg, n_deg, coef_offset;
-  float prior_sigma, log_prior_sigma;
-};
-
-__device__ __forceinline__ int slot_base(const ProposalShape& q, int k) {
-  int b = 0;
-  for (int kk = 0; kk < k; ++kk) b += q.min_deg + kk + q.coef_offset;
-  return b;
-}
-
-__global__ void __launch_bounds__(kTpb) loss_grad_kernel(ProposalShape q,
-                                                         const float* __restrict__ out,
-                                                         const int32_t* __restrict__ n_t,
-                                                         const float* __restrict__ c_t, int32_t B,
-                                                         float* __restrict__ dout,
-                                                         __nv_bfloat16* __restrict__ dout_b,
-                                                         double* loss_sum) {
-  const int b = blockIdx.x * kTpb + threadIdx.x;
-  float loss = 0.0f;
-  if (b < B) {
-    const float* o = out + (int64_t)b * kOut;
-    float g[kOut];
-#pragma unroll
-    for (int i = 0; i < kOut; ++i) g[i] = 0.0f;
-    const int k = n_t[b] - q.min_deg;
-    float mx = -INFINITY;
-    for (int i = 0; i < q.n_deg; ++i) mx = fmaxf(mx, o[i]);
-    float se = 0.0f;
-    for (int i = 0; i < q.n_deg; ++i) se += expf(o[i] - mx);
-    loss = -(o[k] - mx - logf(se));
-    for (int i = 0; i < q.n_deg; ++i) g[i] = expf(o[i] - mx) / se - (i == k ? 1.0f : 0.0f);
-    const int ncoef = n_t[b] + q.coef_offset, base = slot_base(q, k);
-    for (int j = 0; j < ncoef; ++j) {
-      const float om = o[4 + 2 * (base + j)], os = o[5 + 2 * (base + j)];
-      const float t = fminf(fmaxf(os, -9.0f), 1.0f);
-      const float mu = q.prior_sigma * om, sd = q.prior_sigma * expf(t);
-      const float z = (c_t[(int64_t)b * kMaxCoef + j] - mu) / sd;
-      loss += 0.91893853320467274f + q.log_prior_sigma + t + 0.5f * z * z;
-      g[4 + 2 * (base + j)] = -z / sd * q.prior_sigma;
-      g[5 + 2 * (base + j)] = (os > -9.0f && os < 1.0f) ? (1.0f - z * z) : 0.0f;
-    }
-    const float inv = 1.0f / (float)B;
-#pragma unroll
-    for (int i = 0; i < kOut; ++i) {
-      dout[(int64_t)b * kOut + i] = g[i] * inv;
-      dout_b[(int64_t)b * kOut + i] = __float2bfloat16_rn(g[i] * inv);
-    }
-  }
-  loss = warp_sum(loss);
-  __shared__ float red[kTpb / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = loss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.0f;
-    for (int w = 0; w < kTpb / 32; ++w) s += red[w];
-    atomicAdd(loss_sum, (double)s);
-  }
-}
-
-// db[n] = sum over rows of d[m, n] (FP32 or BF16 rows), one thread per column.
-template <typename T>
-__global__ void colsum_kernel(const T* __restrict__ d, int M, int N, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.0f;
-  for (int m = 0; m < M; ++m) {
-    if constexpr (sizeof(T) == 2) s += __bfloat162float(d[(int64_t)m * N + n]);
-    else s += d[(int64_t)m * N + n];
-  }
-  db[n] = s;
+__global__ void __launch_bounds__(kTpb) grad_kernel(const float* __restrict__ partial, int S,
+                                                    float* __restrict__ grad) {
+  const int64_t i = (int64_t)blockIdx.x * kTpb + threadIdx.x;
+  if (i < (int64_t)kNumParams) grad[i] = slice_sum(partial, S, i);
 }
 
 // Adam (Kingma and Ba 2015) on the FP32 master parameters; refreshes the BF16
 // copy of the weights.  step = 1, 2, ... for the bias corrections.
 __global__ void __launch_bounds__(kTpb) adam_kernel(float* __restrict__ p,
-                                                    const float* __restrict__ g,
+                                                    const float* __restrict__ partial, int S,
                                                     float* __restrict__ m, float* __restrict__ v,
                                                     __nv_bfloat16* __restrict__ pb, int64_t n,
                                                     float lr, float b1, float b2, float eps,
@@ -220,7 +124,7 @@ __global__ void __launch_bounds__(kTpb) adam_kernel(float* __restrict__ p,
   const int64_t i = (int64_t)blockIdx.x * kTpb + threadIdx.x;
   if (i >= n) return;
   const float t = (float)(*step);
-  const float gi = g[i];
+  const float gi = slice_sum(partial, S, i);
   const float mi = b1 * m[i] + (1.0f - b1) * gi;
   const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
   m[i] = mi;
@@ -237,118 +141,90 @@ __global__ void to_bf16_kernel(const float* __restrict__ p, __nv_bfloat16* __res
   if (i < n) pb[i] = __float2bfloat16_rn(p[i]);
 }
 
-// The step counter advances; the step's summed loss goes to loss_out[step - 1].
-__global__ void bump_kernel(int32_t* step, const double* loss, double* loss_out) {
-  const int32_t s = *step + 1;
-  *step = s;
-  if (loss_out) loss_out[s - 1] = *loss;
-}
-
 // ---------------------------------------------------------------------------
 // Workspace of the network for a batch of B rows.
 // ---------------------------------------------------------------------------
 struct MlpWs {
   int32_t* status;  // first word: a tensor-core wait that ran out (ppl_workspace_status)
   __nv_bfloat16 *pb, *feat, *h1, *h2, *dout_b, *dh2, *dh1;
-  float *out, *dout, *grad;
+  float *dout, *partial, *warp_loss;
   int32_t* n_t;
   float* c_t;
   double* loss;
   int32_t* step;
-  float* split;  // split-K slices of the products
   size_t total;
 };
 
 static size_t a256(size_t v) { return (v + 255) / 256 * 256; }
 
+// The status word is the workspace's first; the step counter and the loss
+// follow it, and the arrays start at the next 256-byte address, so that the
+// kernels' 16-byte accesses are aligned wherever the caller's workspace lies.
 static MlpWs mlp_ws(char* base, int64_t B) {
+  constexpr size_t kHead = 768;  // the head and the arrays' alignment
+  const size_t start = base ? a256(reinterpret_cast<uintptr_t>(base) + 64) -
+                                  reinterpret_cast<uintptr_t>(base) : 0;
   MlpWs w;
   size_t off = 0;
   auto take = [&](size_t bytes) {
-    char* p = base ? base + off : nullptr;
+    char* p = base ? base + start + off : nullptr;
     off += a256(bytes);
     return p;
   };
-  w.status = (int32_t*)take(sizeof(int32_t));
-  w.step = (int32_t*)take(sizeof(int32_t));
-  w.loss = (double*)take(sizeof(double) * 2);
+  // 8-byte aligned, past the status word
+  char* head = base ? reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(base) + 4 + 7) / 8 * 8)
+                    : nullptr;
+  w.status = reinterpret_cast<int32_t*>(base);
+  w.loss = reinterpret_cast<double*>(head);
+  w.step = reinterpret_cast<int32_t*>(head ? head + 8 : nullptr);
   w.pb = (__nv_bfloat16*)take(kNumParams * 2);
-  w.grad = (float*)take(kNumParams * 4);
   w.feat = (__nv_bfloat16*)take(B * kIn * 2);
   w.h1 = (__nv_bfloat16*)take(B * kHid * 2);
   w.h2 = (__nv_bfloat16*)take(B * kHid * 2);
-  w.out = (float*)take(B * kOut * 4);
   w.dout = (float*)take(B * kOut * 4);
   w.dout_b = (__nv_bfloat16*)take(B * kOut * 2);
   w.dh2 = (__nv_bfloat16*)take(B * kHid * 2);
   w.dh1 = (__nv_bfloat16*)take(B * kHid * 2);
   w.n_t = (int32_t*)take(B * 4);
   w.c_t = (float*)take(B * kMaxCoef * 4);
-  w.split = (float*)take(kSplitFloats * 4);
-  w.total = off;
+  w.warp_loss = (float*)take((size_t)((B + 127) / 128) * 4 * 4);
+  w.partial = (float*)take((size_t)kDwSlices * kNumParams * 4);
+  w.total = off + kHead;
   return w;
 }
 
-static cudaError_t mlp_forward(const float* params, const MlpWs& w, int B, cudaStream_t s) {
-  GemmArgs g{};
-  g.A = w.feat; g.sam = kIn; g.sak = 1;
-  g.B = w.pb + kOffW1; g.sbn = kIn; g.sbk = 1;
-  g.M = B; g.N = kHid; g.K = kIn; g.bias = params + kOffB1; g.relu = 1; g.Cb = w.h1;
-  cudaError_t e = gemm(g, w.status, s, w.split);
-  if (e != cudaSuccess) return e;
-  g = GemmArgs{};
-  g.A = w.h1; g.sam = kHid; g.sak = 1;
-  g.B = w.pb + kOffW2; g.sbn = kHid; g.sbk = 1;
-  g.M = B; g.N = kHid; g.K = kHid; g.bias = params + kOffB2; g.relu = 1; g.Cb = w.h2;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  g = GemmArgs{};
-  g.A = w.h2; g.sam = kHid; g.sak = 1;
-  g.B = w.pb + kOffW3; g.sbn = kHid; g.sbk = 1;
-  g.M = B; g.N = kOut; g.K = kHid; g.bias = params + kOffB3; g.Cf = w.out;
-  return gemm(g, w.status, s, w.split);
+static NetArgs net_args(const float* params, const MlpWs& w, int B) {
+  NetArgs a{};
+  a.params = params;
+  a.pb = w.pb;
+  a.feat = w.feat;
+  a.B = B;
+  a.status = w.status;
+  return a;
 }
 
-// Gradient of the mean loss over the batch into w.grad (FP32), loss sum into w.loss[0].
-static cudaError_t mlp_backward(const ProposalShape& q, const MlpWs& w, int B, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(w.loss, 0, sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  loss_grad_kernel<<<(B + kTpb - 1) / kTpb, kTpb, 0, s>>>(q, w.out, w.n_t, w.c_t, B, w.dout,
-                                                         w.dout_b, w.loss);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  GemmArgs g{};
-  // dW3[o, i] = sum_b dout[b, o] h2[b, i]
-  g.A = w.dout_b; g.sam = 1; g.sak = kOut;
-  g.B = w.h2; g.sbn = 1; g.sbk = kHid;
-  g.M = kOut; g.N = kHid; g.K = B; g.Cf = w.grad + kOffW3;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  colsum_kernel<float><<<1, 64, 0, s>>>(w.dout, B, kOut, w.grad + kOffB3);
-  // dh2[b, i] = sum_o dout[b, o] W3[o, i], masked by h2 > 0
-  g = GemmArgs{};
-  g.A = w.dout_b; g.sam = kOut; g.sak = 1;
-  g.B = w.pb + kOffW3; g.sbn = 1; g.sbk = kHid;
-  g.M = B; g.N = kHid; g.K = kOut; g.mask = w.h2; g.Cb = w.dh2;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  // dW2[o, i] = sum_b dh2[b, o] h1[b, i]
-  g = GemmArgs{};
-  g.A = w.dh2; g.sam = 1; g.sak = kHid;
-  g.B = w.h1; g.sbn = 1; g.sbk = kHid;
-  g.M = kHid; g.N = kHid; g.K = B; g.Cf = w.grad + kOffW2;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  colsum_kernel<__nv_bfloat16><<<1, kHid, 0, s>>>(w.dh2, B, kHid, w.grad + kOffB2);
-  // dh1 = (dh2 W2) masked by h1 > 0
-  g = GemmArgs{};
-  g.A = w.dh2; g.sam = kHid; g.sak = 1;
-  g.B = w.pb + kOffW2; g.sbn = 1; g.sbk = kHid;
-  g.M = B; g.N = kHid; g.K = kHid; g.mask = w.h1; g.Cb = w.dh1;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  // dW1[o, i] = sum_b dh1[b, o] feat[b, i]
-  g = GemmArgs{};
-  g.A = w.dh1; g.sam = 1; g.sak = kHid;
-  g.B = w.feat; g.sbn = 1; g.sbk = kIn;
-  g.M = kHid; g.N = kIn; g.K = B; g.Cf = w.grad + kOffW1;
-  if ((e = gemm(g, w.status, s, w.split)) != cudaSuccess) return e;
-  colsum_kernel<__nv_bfloat16><<<1, kHid, 0, s>>>(w.dh1, B, kHid, w.grad + kOffB1);
-  return cudaGetLastError();
+// Forward, loss and gradients of B pairs (w.feat, w.n_t, w.c_t): the weight
+// gradients' slices into w.partial, the summed loss into *w.loss.
+static cudaError_t mlp_backward(const float* params, const ProposalShape& q, const MlpWs& w, int B,
+                                int32_t* step, double* loss_out, cudaStream_t s) {
+  NetArgs a = net_args(params, w, B);
+  a.backward = 1;
+  a.shape = q;
+  a.n_t = w.n_t;
+  a.c_t = w.c_t;
+  a.h1 = w.h1;
+  a.h2 = w.h2;
+  a.dh2 = w.dh2;
+  a.dh1 = w.dh1;
+  a.dout = w.dout;
+  a.dout_b = w.dout_b;
+  a.warp_loss = w.warp_loss;
+  a.partial = w.partial;
+  a.loss = w.loss;
+  a.step = step;
+  a.loss_out = loss_out;
+  const cudaError_t e = launch_net(a, s);
+  return e != cudaSuccess ? e : launch_dw(a, s);
 }
 
 static ProposalShape shape_of(const PolyParams& p, float prior_sigma) {
@@ -413,8 +289,9 @@ ppl_status ppl_proposal_forward(const ppl_model* model, const float* params, con
                                                                             kNumParams);
   features_kernel<<<(unsigned)(((int64_t)n_sets * 32 + kTpb - 1) / kTpb), kTpb, 0, s>>>(
       x, y, n_sets, w.feat);
-  w.out = out_dev;
-  return st(mlp_forward(params, w, n_sets, s));
+  NetArgs a = net_args(params, w, n_sets);
+  a.out = out_dev;
+  return st(launch_net(a, s));
 }
 
 ppl_status ppl_proposal_features(const float* x, const float* y, int32_t n_sets, void* feat_dev,
@@ -441,16 +318,13 @@ ppl_status ppl_proposal_grad(const ppl_model* model, const float* params, int64_
                                                                             kNumParams);
   forward_sim_kernel<<<(unsigned)(((int64_t)batch * 32 + kTpb - 1) / kTpb), kTpb, 0, s>>>(
       p, model->obs_sigma, seed, pair0, batch, w.feat, w.n_t, w.c_t);
-  ppl_status r = st(mlp_forward(params, w, batch, s));
+  w.loss = loss_out;
+  const ppl_status r = st(mlp_backward(params, shape_of(p, model->prior_sigma), w, batch, nullptr,
+                                       nullptr, s));
   if (r != PPL_OK) return r;
-  r = st(mlp_backward(shape_of(p, model->prior_sigma), w, batch, s));
-  if (r != PPL_OK) return r;
-  if (cudaMemcpyAsync(grad_out, w.grad, kNumParams * sizeof(float), cudaMemcpyDeviceToDevice,
-                      s) != cudaSuccess ||
-      cudaMemcpyAsync(loss_out, w.loss, sizeof(double), cudaMemcpyDeviceToDevice, s) !=
-          cudaSuccess)
-    return PPL_ECUDA;
-  return PPL_OK;
+  grad_kernel<<<(unsigned)((kNumParams + kTpb - 1) / kTpb), kTpb, 0, s>>>(
+      w.partial, dw_slices(batch), grad_out);
+  return st(cudaGetLastError());
 }
 
 ppl_status ppl_proposal_train_init(const float* params, int32_t batch, void* ws,
@@ -484,13 +358,11 @@ ppl_status ppl_proposal_train_steps(const ppl_model* model, float* params, float
   for (int32_t it = 0; it < n_steps; ++it) {
     forward_sim_kernel<<<(unsigned)(((int64_t)batch * 32 + kTpb - 1) / kTpb), kTpb, 0, s>>>(
         p, model->obs_sigma, seed, 0, batch, w.feat, w.n_t, w.c_t, w.step, steps_per_epoch);
-    ppl_status r = st(mlp_forward(params, w, batch, s));
+    const ppl_status r = st(mlp_backward(params, q, w, batch, w.step, loss_per_step, s));
     if (r != PPL_OK) return r;
-    r = st(mlp_backward(q, w, batch, s));
-    if (r != PPL_OK) return r;
-    bump_kernel<<<1, 1, 0, s>>>(w.step, w.loss, loss_per_step);
     adam_kernel<<<(unsigned)((kNumParams + kTpb - 1) / kTpb), kTpb, 0, s>>>(
-        params, w.grad, adam_m, adam_v, w.pb, kNumParams, lr, 0.9f, 0.999f, 1e-8f, w.step);
+        params, w.partial, dw_slices(batch), adam_m, adam_v, w.pb, kNumParams, lr, 0.9f, 0.999f,
+        1e-8f, w.step);
   }
   return st(cudaGetLastError());
 }

@@ -1,0 +1,56 @@
+// The proposal network's shapes and the arguments shared by its kernels.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "common.cuh"
+
+namespace ppl {
+
+constexpr int kIn = 64, kHid = 256, kOut = 48, kPts = 32;
+// parameter buffer layout (FP32, and its BF16 copy): W1 | b1 | W2 | b2 | W3 | b3
+constexpr size_t kOffW1 = 0, kOffB1 = kOffW1 + kHid * kIn, kOffW2 = kOffB1 + kHid,
+                 kOffB2 = kOffW2 + kHid * kHid, kOffW3 = kOffB2 + kHid,
+                 kOffB3 = kOffW3 + kOut * kHid, kNumParams = kOffB3 + kOut;
+constexpr int kDwSlices = 4;  // most batch slices of the weight gradients (8: 57 us a step against 59)
+
+struct ProposalShape {
+  int min_deg, n_deg, coef_offset;
+  float prior_sigma, log_prior_sigma;
+};
+
+__device__ __forceinline__ int slot_base(const ProposalShape& q, int k) {
+  int b = 0;
+  for (int kk = 0; kk < k; ++kk) b += q.min_deg + kk + q.coef_offset;
+  return b;
+}
+
+// One pass of the network over B pairs (or data sets, forward only).  16-byte
+// aligned: pb, feat, the activations and their gradients, dout, dout_b, partial.
+struct NetArgs {
+  const float* params;       // biases are read from the FP32 parameters
+  const __nv_bfloat16* pb;   // BF16 copy of the parameters
+  const __nv_bfloat16* feat; // [B][64]
+  int B;
+  int backward;
+  int slices_hid, slices_out;
+  float* out;                // [B][48] FP32, or null
+  ProposalShape shape;
+  const int32_t* n_t;        // [B] degrees
+  const float* c_t;          // [B][6] coefficients
+  __nv_bfloat16 *h1, *h2, *dh2, *dh1;  // [B][256], null when not wanted
+  float* dout;               // [B][48]
+  __nv_bfloat16* dout_b;     // [B][48]
+  float* warp_loss;          // [ceil(B / 128) 4] sums of 32 pairs' losses
+  float* partial;            // [slices][kNumParams] weight-gradient slices
+  double* loss;              // the batch's summed loss, or null
+  int32_t* step;             // training: device step counter, advanced, or null
+  double* loss_out;          // training: loss of step s at [s], or null
+  int32_t* status;
+};
+
+cudaError_t launch_net(NetArgs a, cudaStream_t s);
+cudaError_t launch_dw(const NetArgs& a, cudaStream_t s);
+int dw_slices(int64_t B);
+
+}  // namespace ppl

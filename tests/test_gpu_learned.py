@@ -206,3 +206,29 @@ def test_training_steps_replayed_from_a_cuda_graph_match_direct_training(ppl):
     assert ppl.ppl_workspace_status(ws) == 0
     assert torch.equal(pb, pa) and torch.equal(mb, ma) and torch.equal(vb, va)
     assert torch.allclose(lb, la, rtol=1e-12, atol=0.0)
+
+
+@pytest.mark.parametrize("B", [1, 63, 129, 700, 2049])
+def test_gradient_at_tile_edges(ppl, mlp, orc, B):
+    # ragged tiles of 128 pairs and batch slices of 64; a workspace 8 bytes off
+    # its allocation's alignment gives the same bits
+    import torch
+    W = synth.mlp_weights(8, bias_scale=0.3)
+    m = orc.poly_model()
+    params = ppl.pack_params(W)
+    grad, loss = ppl.ppl_proposal_grad(ppl.poly_model(), params, 100, B, 21)
+    ws = torch.empty(ppl.proposal_workspace(B).numel() + 8, dtype=torch.uint8, device="cuda")[8:]
+    grad2, loss2 = ppl.ppl_proposal_grad(ppl.poly_model(), params, 100, B, 21, ws=ws)
+    assert torch.equal(grad, grad2) and torch.equal(loss, loss2)
+    assert ppl.ppl_workspace_status(ws) == 0
+    pairs = [mlp.forward_sim(m, 21, 100 + p) for p in range(B)]
+    feats = np.stack([mlp.features(x, y) for x, y, _, _ in pairs])
+    ref_loss, g = mlp.loss_grad(m, W, feats, np.array([p[2] for p in pairs]),
+                                np.stack([p[3] for p in pairs]))
+    assert float(loss.item()) / B == pytest.approx(ref_loss, rel=2e-3)
+    flat, off = grad.cpu().numpy(), 0
+    for gi in g:
+        got = flat[off:off + gi.size].reshape(gi.shape)
+        off += gi.size
+        # the bound of BF16 operands; a single pair's products do not average
+        assert np.linalg.norm(got - gi) <= (3e-2 if B > 1 else 6e-2) * np.linalg.norm(gi) + 1e-12
