@@ -198,6 +198,9 @@ ppl_status ppl_infer_is_suffstat(const ppl_model* model, const ppl_data* data,
   // the statistics live in the scratch region, unused by likelihood weighting
   const int d_max = p.min_deg + p.n_deg - 1 + p.coef_offset;
   PPL_TRY(cuda_status(launch_suffstat(data->x, data->y, data->len, d_max, w.scratch(), s)));
+  PPL_TRY(cuda_status(launch_suffstat_trace(p, w.scratch(), n_particles, seed, instance, lw_out,
+                                            particles_out, w.hdr(), w.partials(), out_dev, s)));
+  // the point-by-point sum, when the Gram matrix is singular to working precision
   PPL_TRY(cuda_status(launch_poly_trace(p, data->x, data->y, data->len, n_particles, seed,
                                         instance, lw_out, particles_out, w.hdr(), w.partials(),
                                         out_dev, s, w.scratch())));

@@ -28,10 +28,11 @@ int stream_grid(int64_t N);
 size_t partials_bytes();
 
 // is_kernels.cu
+// unless_ok (sufficient statistics, optional): run only when these are not ok.
 cudaError_t launch_poly_trace(const PolyParams& p, const float* x, const float* y, int64_t L,
                               int64_t N, uint64_t seed, uint32_t instance, float* lw_out,
                               ppl_poly_particle* rec_out, WsHeader* hdr, void* parts,
-                              ppl_is_result* res, cudaStream_t s, const void* suff = nullptr);
+                              ppl_is_result* res, cudaStream_t s, const void* unless_ok = nullptr);
 // trace_tc.cu: the same pass with the factor's polynomial evaluations on the
 // tensor cores (data sets of up to trace_tc_max_points() points).
 // With part_out, the shard partial of particles [first, first + N) of a
@@ -60,6 +61,10 @@ cudaError_t launch_discrete_is(int32_t model, const int32_t* data, int64_t n_dat
                                ppl_discrete_result* res, cudaStream_t s);
 cudaError_t launch_suffstat(const float* x, const float* y, int64_t L, int d_max, void* out,
                             cudaStream_t s);
+// The likelihood-weighting pass on them (nothing when they are not ok).
+cudaError_t launch_suffstat_trace(const PolyParams& p, const void* stat, int64_t N, uint64_t seed,
+                                  uint32_t instance, float* lw_out, ppl_poly_particle* rec_out,
+                                  WsHeader* hdr, void* parts, ppl_is_result* res, cudaStream_t s);
 cudaError_t launch_stats(const float* lw, int64_t N, WsHeader* hdr, void* parts,
                          double* lse_out, cudaStream_t s);
 cudaError_t launch_posterior(const PolyParams& p, const ppl_poly_particle* rec, const float* lw,

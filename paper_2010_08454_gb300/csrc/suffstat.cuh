@@ -25,9 +25,10 @@ struct SuffStat {
 };
 
 // The sum of squared residuals of a trace with d coefficients (c_j = 0 for j >= d).
-__device__ __forceinline__ float suff_residual(const SuffStat& s, const float (&c)[kMaxCoef],
-                                               int d) {
-  float ss = s.base[d];
+// (`base` is s.base where it can be indexed; s.R and s.w stay in registers)
+__device__ __forceinline__ float suff_residual(const SuffStat& s, const float* base,
+                                               const float (&c)[kMaxCoef], int d) {
+  float ss = base[d];
 #pragma unroll
   for (int i = 0; i < kMaxCoef; ++i) {
     if (i < d) {

@@ -14,7 +14,6 @@
 #pragma once
 
 #include "posterior.cuh"
-#include "suffstat.cuh"
 
 namespace ppl {
 
@@ -354,6 +353,115 @@ struct PriorDraw {
   }
 };
 
+// Fold the warp's traces (one per lane: log-weight, degree index d in [0, 4)
+// or -1, global index, coefficients) into the warp's running per-degree
+// partials.  A trace more than kSkipNats below its degree's running
+// maximum carries a weight below e^-50 of it and is skipped; NaN log-weights
+// only raise the flag.
+__device__ __forceinline__ void fold_warp(DegPartial* wr, float lw, int d, int idx,
+                                          const float (&c)[kMaxCoef], int lane, int& nan) {
+  float thr = -INFINITY;
+#pragma unroll
+  for (int k = 0; k < kMaxDegrees; ++k)
+    if (d == k) thr = wr[k].m - kSkipNats;
+  const bool is_nan = d >= 0 && lw != lw;
+  nan |= is_nan;
+  bool cand = d >= 0 && !is_nan && lw > thr;
+  unsigned cm = __ballot_sync(0xffffffffu, cand);
+  if (!cm) return;
+  if (__popc(cm) > kSerialMerges) {
+    // many traces above the running thresholds (a warp's first tiles): a
+    // trace more than kSkipNats below the best of its degree in this tile
+    // is negligible as well
+    float tmax = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kMaxDegrees; ++k) {
+      float m = (cand && d == k) ? lw : -INFINITY;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (d == k) tmax = m;
+    }
+    cand = cand && lw > tmax - kSkipNats;
+    cm = __ballot_sync(0xffffffffu, cand);
+  }
+  if (__popc(cm) <= kSerialMerges) {
+    while (cm) {
+      const int src = __ffs(cm) - 1;
+      cm &= cm - 1;
+      const float v = __shfl_sync(0xffffffffu, lw, src);
+      const int dv = __shfl_sync(0xffffffffu, d, src);
+      const int iv = __shfl_sync(0xffffffffu, idx, src);
+      float cc[kMaxCoef];
+#pragma unroll
+      for (int k = 0; k < kMaxCoef; ++k) cc[k] = __shfl_sync(0xffffffffu, c[k], src);
+      if (lane == 0) {
+        DegPartial p;
+        deg_empty(p);
+        p.m = v;
+        p.arg = iv;
+        if (v > -INFINITY) {
+          p.S = 1.0f;
+          p.S2 = 1.0f;
+#pragma unroll
+          for (int k = 0; k < kMaxCoef; ++k) p.mean[k] = cc[k];
+        }
+        deg_merge(wr[dv], p);
+      }
+      __syncwarp();
+    }
+    return;
+  }
+  for (int dd = 0; dd < kMaxDegrees; ++dd) {
+    const bool mine = cand && d == dd;
+    if (!__any_sync(0xffffffffu, mine)) continue;
+    float m = mine ? lw : -INFINITY;
+    int a = mine ? idx : 0x7fffffff, src = lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, m, o);
+      const int oa = __shfl_xor_sync(0xffffffffu, a, o);
+      const int os = __shfl_xor_sync(0xffffffffu, src, o);
+      if (om > m || (om == m && oa < a)) {
+        m = om;
+        a = oa;
+        src = os;
+      }
+    }
+    if (!(m > -INFINITY)) continue;  // only -inf traces of this degree
+    float ref[kMaxCoef];
+#pragma unroll
+    for (int k = 0; k < kMaxCoef; ++k) ref[k] = __shfl_sync(0xffffffffu, c[k], src);
+    const float w = (mine && lw > -INFINITY) ? expf(lw - m) : 0.0f;
+    const float S = warp_sum(w), S2 = warp_sum(w * w);
+    float A[kMaxCoef], B[kMaxCoef];
+#pragma unroll
+    for (int k = 0; k < kMaxCoef; ++k) {
+      const float dc = mine ? c[k] - ref[k] : 0.0f;
+      const float t = w * dc;
+      A[k] = warp_sum(t);
+      B[k] = warp_sum(t * dc);
+    }
+    if (lane == 0) {
+      DegPartial p;
+      deg_empty(p);
+      p.m = m;
+      p.arg = a;
+      p.S = S;
+      p.S2 = S2;
+      if (S > 0.0f) {
+#pragma unroll
+        for (int k = 0; k < kMaxCoef; ++k) {
+          const float sh = A[k] / S;
+          p.mean[k] = ref[k] + sh;
+          p.M2[k] = fmaxf(B[k] - sh * A[k], 0.0f);
+        }
+      }
+      deg_merge(wr[dd], p);
+    }
+    __syncwarp();
+  }
+}
+
 // A warp's candidates for its per-degree partials (phase C of trace_group).
 template <int PPT>
 struct Cands {
@@ -464,7 +572,7 @@ __device__ __forceinline__ void trace_group(const Draw& draw, const PolyParams& 
                                             bool resident, float2* sdata, int64_t N,
                                             int64_t base, float* __restrict__ lw_out,
                                             ppl_poly_particle* __restrict__ rec_out,
-                                            TraceSmem<PPT>& ts, const SuffStat* suff = nullptr) {
+                                            TraceSmem<PPT>& ts) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const bool rec_v8 = (reinterpret_cast<uintptr_t>(rec_out) & 31) == 0;
@@ -565,13 +673,7 @@ __device__ __forceinline__ void trace_group(const Draw& draw, const PolyParams& 
       }
     }
   }
-  if (suff != nullptr && suff->ok) {  // the same branch for the whole block
-    // sufficient statistics: O(d^2) per trace, d its own coefficient count
-#pragma unroll
-    for (int j = 0; j < PPT; ++j)
-      if (slot[j] < n_valid)
-        ss[j] = suff_residual(*suff, c[j], p.min_deg + slot_degree(ts.off, slot[j]) + p.coef_offset);
-  } else if (resident) {
+  if (resident) {
     accumulate_rows<PPT>(nc, sdata, (int)L, c, ss, comp);
   } else {
     for (int64_t l0 = 0; l0 < L; l0 += chunk) {

@@ -55,8 +55,6 @@ constexpr int kTcChunk = 128;       // data points per product (MMA N): 512 colu
 constexpr int kTcThreads = 128 * kTcWGs;
 constexpr int kTcSpin = 1 << 18;    // bound of one mbarrier wait (polls)
 constexpr uint32_t kTcSuspendNs = 4096;  // a poll may suspend the warp this long (hint)
-constexpr float kTcSkipNats = 50.0f;
-constexpr int kTcSerialMerges = 4;  // up to this many traces a warp merges one at a time
 constexpr uint32_t kTcTmemCols = 512;
 constexpr int kTcMaxPoints = 2048;  // the data's B operand (64 B per point) stays in shared memory
 
@@ -141,15 +139,6 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// One 32-byte record in a single 256-bit store (p 32-byte aligned).
-__device__ __forceinline__ void st_record_v8(void* p, const float (&c)[kMaxCoef], int n,
-                                             uint32_t i) {
-  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(c[0]),
-               "f"(c[1]), "f"(c[2]), "f"(c[3]), "f"(c[4]), "f"(c[5]), "f"(__int_as_float(n)),
-               "f"(__uint_as_float(i))
-               : "memory");
-}
-
 struct TcShared {
   DegPartial wrun[(kTcThreads / 32) * kMaxDegrees];  // each warp's running per-degree partials
   uint64_t mbar[kTcWGs];
@@ -202,115 +191,6 @@ __device__ __forceinline__ bool issue_chunk(int g, int r, uint32_t tmem_d, uint3
                  : "memory");
   }
   return false;
-}
-
-// Fold the warp's traces (one per lane: log-weight, degree index d in [0, 4)
-// or -1, global index, coefficients) into the warp's running per-degree
-// partials.  A trace more than kTcSkipNats below its degree's running
-// maximum carries a weight below e^-50 of it and is skipped; NaN log-weights
-// only raise the flag.
-__device__ __forceinline__ void fold_warp(DegPartial* wr, float lw, int d, int idx,
-                                          const float (&c)[kMaxCoef], int lane, int& nan) {
-  float thr = -INFINITY;
-#pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k)
-    if (d == k) thr = wr[k].m - kTcSkipNats;
-  const bool is_nan = d >= 0 && lw != lw;
-  nan |= is_nan;
-  bool cand = d >= 0 && !is_nan && lw > thr;
-  unsigned cm = __ballot_sync(0xffffffffu, cand);
-  if (!cm) return;
-  if (__popc(cm) > kTcSerialMerges) {
-    // many traces above the running thresholds (a warp's first tiles): a
-    // trace more than kTcSkipNats below the best of its degree in this tile
-    // is negligible as well
-    float tmax = -INFINITY;
-#pragma unroll
-    for (int k = 0; k < kMaxDegrees; ++k) {
-      float m = (cand && d == k) ? lw : -INFINITY;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (d == k) tmax = m;
-    }
-    cand = cand && lw > tmax - kTcSkipNats;
-    cm = __ballot_sync(0xffffffffu, cand);
-  }
-  if (__popc(cm) <= kTcSerialMerges) {
-    while (cm) {
-      const int src = __ffs(cm) - 1;
-      cm &= cm - 1;
-      const float v = __shfl_sync(0xffffffffu, lw, src);
-      const int dv = __shfl_sync(0xffffffffu, d, src);
-      const int iv = __shfl_sync(0xffffffffu, idx, src);
-      float cc[kMaxCoef];
-#pragma unroll
-      for (int k = 0; k < kMaxCoef; ++k) cc[k] = __shfl_sync(0xffffffffu, c[k], src);
-      if (lane == 0) {
-        DegPartial p;
-        deg_empty(p);
-        p.m = v;
-        p.arg = iv;
-        if (v > -INFINITY) {
-          p.S = 1.0f;
-          p.S2 = 1.0f;
-#pragma unroll
-          for (int k = 0; k < kMaxCoef; ++k) p.mean[k] = cc[k];
-        }
-        deg_merge(wr[dv], p);
-      }
-      __syncwarp();
-    }
-    return;
-  }
-  for (int dd = 0; dd < kMaxDegrees; ++dd) {
-    const bool mine = cand && d == dd;
-    if (!__any_sync(0xffffffffu, mine)) continue;
-    float m = mine ? lw : -INFINITY;
-    int a = mine ? idx : 0x7fffffff, src = lane;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, m, o);
-      const int oa = __shfl_xor_sync(0xffffffffu, a, o);
-      const int os = __shfl_xor_sync(0xffffffffu, src, o);
-      if (om > m || (om == m && oa < a)) {
-        m = om;
-        a = oa;
-        src = os;
-      }
-    }
-    if (!(m > -INFINITY)) continue;  // only -inf traces of this degree
-    float ref[kMaxCoef];
-#pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) ref[k] = __shfl_sync(0xffffffffu, c[k], src);
-    const float w = (mine && lw > -INFINITY) ? expf(lw - m) : 0.0f;
-    const float S = warp_sum(w), S2 = warp_sum(w * w);
-    float A[kMaxCoef], B[kMaxCoef];
-#pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) {
-      const float dc = mine ? c[k] - ref[k] : 0.0f;
-      const float t = w * dc;
-      A[k] = warp_sum(t);
-      B[k] = warp_sum(t * dc);
-    }
-    if (lane == 0) {
-      DegPartial p;
-      deg_empty(p);
-      p.m = m;
-      p.arg = a;
-      p.S = S;
-      p.S2 = S2;
-      if (S > 0.0f) {
-#pragma unroll
-        for (int k = 0; k < kMaxCoef; ++k) {
-          const float sh = A[k] / S;
-          p.mean[k] = ref[k] + sh;
-          p.M2[k] = fmaxf(B[k] - sh * A[k], 0.0f);
-        }
-      }
-      deg_merge(wr[dd], p);
-    }
-    __syncwarp();
-  }
 }
 
 }  // namespace
@@ -411,7 +291,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) poly_trace_tc_kernel(
     nn = draw(gi, cc, corr);
     if (i < N && rec_out) {
       if (rec_v8) {
-        st_record_v8(rec_out + i, cc, nn, gi);
+        st_global_v8(rec_out + i, cc[0], cc[1], cc[2], cc[3], cc[4], cc[5], __int_as_float(nn),
+                     __uint_as_float(gi));
       } else {
         float4* dst = reinterpret_cast<float4*>(rec_out + i);
         dst[0] = make_float4(cc[0], cc[1], cc[2], cc[3]);

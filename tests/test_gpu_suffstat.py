@@ -53,3 +53,20 @@ def test_suffstat_other_readings(ppl, orc):
                dict(min_deg=1, max_deg=1)]:
         (res, lw, n, c, origin), _ = _both(ppl, x, y, 20000, 11, **kw)
         check_is(orc, res, lw, n, c, origin, x, y, 20000, 11, kw)
+
+
+@pytest.mark.parametrize("N", [1, 31, 33, 64, 65, 511, 513, 155647, 155649])
+def test_suffstat_population_edges(ppl, orc, N):
+    # warps of 64 traces, blocks of 512, 304 blocks: one more or less of each
+    x, y = synth.poly_dataset(40, 3)
+    (res, lw, n, c, origin), _ = _both(ppl, x, y, N, 17)
+    check_is(orc, res, lw, n, c, origin, x, y, N, 17, {})
+
+
+def test_suffstat_reports_nan(ppl):
+    import torch
+    x, y = (torch.from_numpy(v).cuda() for v in synth.poly_dataset(40, 3))
+    y[7] = float("nan")
+    ws = ppl.workspace(ppl.poly_model(), 3000, 40)
+    ppl.ppl_infer_is_suffstat(ppl.poly_model(), x, y, 3000, 1, ws=ws)
+    assert ppl.ppl_workspace_status(ws) == ppl.PPL_ENAN
