@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "lanesums.cuh"
 #include "learned.cuh"
 #include "posterior.cuh"
 #include "trace.cuh"
@@ -61,6 +62,30 @@ static BatchLayout batch_layout(int64_t n_items, int32_t n_inst) {
   return l;
 }
 
+// The summary of an instance from its `tiles` tiles' partials, by one block.
+__device__ __forceinline__ void finish_instance(const PolyParams& p, const DegPartial* parts,
+                                                int64_t tiles, int64_t N, WsHeader* hdr,
+                                                ppl_is_result* out) {
+  __shared__ DegPartial fin[kMaxDegrees];
+  __shared__ float2 fS[kMaxDegrees], fS2[kMaxDegrees];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < kMaxDegrees) {  // (tile, warp) partials of degree `warp`
+    DegPartial a;
+    DegSums ds;
+    merge_degree(parts, (int)(tiles * (kTpb / 32)), warp, lane, a, ds);
+    if (lane == 0) {
+      fin[warp] = a;
+      fS[warp] = ds.S;
+      fS2[warp] = ds.S2;
+    }
+  }
+  __syncthreads();
+  if (warp == 0)
+    write_summary_warp(fin, fS, fS2, p.n_deg, p.min_deg, N,
+                       lane == 0 ? ld_volatile_i32(&hdr->status) : 0, out);
+  __syncthreads();
+}
+
 constexpr int kBatchChunk = 4096;  // data points staged in shared memory at a time
 
 template <int PPT, bool LEARNED>
@@ -73,8 +98,6 @@ __global__ void __launch_bounds__(kTpb, PPT >= 8 ? 2 : (LEARNED ? 3 : 4)) batche
   extern __shared__ __align__(16) unsigned char smem[];
   TraceSmem<PPT>& ts = *reinterpret_cast<TraceSmem<PPT>*>(smem);
   float2* sdata = reinterpret_cast<float2*>(smem + trace_smem_bytes<PPT>());
-  __shared__ DegPartial gout[kMaxDegrees], fin[kMaxDegrees];
-  __shared__ float2 fS[kMaxDegrees], fS2[kMaxDegrees];
   __shared__ int64_t item_sh;
   __shared__ bool last_sh;
   __shared__ ProposalSmem prop;
@@ -110,7 +133,7 @@ __global__ void __launch_bounds__(kTpb, PPT >= 8 ? 2 : (LEARNED ? 3 : 4)) batche
     if (LEARNED) {
       if (b != cur_prop) {
         __syncthreads();
-        if (tid == 0) load_proposal(p, proposal + (int64_t)b * 48, prop);
+        if (warp == 0) load_proposal(p, proposal + (int64_t)b * 48, prop);
         __syncthreads();
         cur_prop = b;
       }
@@ -149,32 +172,242 @@ __global__ void __launch_bounds__(kTpb, PPT >= 8 ? 2 : (LEARNED ? 3 : 4)) batche
     __syncthreads();
     if (last_sh) {
       __threadfence();
-      const int64_t i0 = first[b];
       const int64_t ni = (N + (int64_t)kTpb * PPT - 1) / ((int64_t)kTpb * PPT);
-      const int64_t np = ni * (kTpb / 32);  // (tile, warp) partials per degree
-      if (warp < kMaxDegrees) {
-        DegPartial a;
-        DegSums ds;
-        merge_degree(parts + i0 * (kTpb / 32) * kMaxDegrees, (int)np, warp, lane, a, ds);
-        if (lane == 0) {
-          fin[warp] = a;
-          fS[warp] = ds.S;
-          fS2[warp] = ds.S2;
-        }
+      finish_instance(p, parts + (int64_t)first[b] * kWarpParts, ni, N, hdr, out + b);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Short data sets.  With a few dozen points the factor is no longer what a
+// trace costs: the degree sort is (about 150 instructions a trace with its
+// shared-memory round trip and barriers), and under a learned proposal, whose
+// weights are nearly even, the fold of nearly every trace by warp reductions
+// (70 shuffles per degree present in a warp's 256 traces).  Here a thread keeps
+// its traces to itself: two at a time, Horner chains padded to six
+// coefficients as f32x2 pairs (the same log-weights, bit for bit: padding adds
+// exact zeros), and lane sums of all four degrees in registers
+// (lanesums.cuh), reduced once per run of tiles.
+//
+// A block takes runs of consecutive tiles of one instance from the queue, in
+// instance order, and leaves one partial per warp in the run's first slot
+// (empty ones in the others).  A warp's reference is the best of its first
+// traces and moves when a trace lies kRebaseNats above it; nothing a run
+// computes depends on the other runs, so the result does not depend on timing.
+//
+// 1024 sets x 2^16 traces, 32 points, sorted kernel and this one: 3160 and 2050
+// us under near-posterior proposals, 1700 and 1640 us with prior draws, 1720
+// and 1380 us on 16 points.  A run costs about 13 us of a block besides its
+// traces (the first traces' references, the reduction), so the line lies
+// where runs of 16384 traces fill the blocks several times over; below it
+// prior draws lose (300 x 100000: 755 and 794 us), and above 32 points too,
+// where the padded chains outweigh the sort (64 points: 1055 and 1160 us).
+// Both draws take the same kernel, so that a proposal equal to the prior gives
+// the prior's run bit for bit.
+// ---------------------------------------------------------------------------
+constexpr int kLanesMaxLen = 32;  // a multiple of 16
+constexpr int64_t kRunTraces = 16384, kLanesMinMean = kRunTraces, kLanesMinTotal = (int64_t)1 << 25;
+
+struct __align__(16) LaneRef {
+  float v[kMaxDegrees][8];  // ref c[6], m_ref, the best log-weight so far
+  int arg[kMaxDegrees];     // and its trace
+};
+
+template <bool LEARNED>
+__global__ void __launch_bounds__(kTpb, 2) lanes_kernel(
+    PolyParams p, const float* __restrict__ xs, const float* __restrict__ ys,
+    const int64_t* __restrict__ data_off, const int64_t* __restrict__ part_off, int n_inst,
+    int64_t n_tiles, int tile_traces, int run_tiles, const int32_t* __restrict__ first,
+    int32_t* count, uint64_t seed, const float* __restrict__ proposal, WsHeader* hdr,
+    DegPartial* parts, ppl_is_result* out) {
+  __shared__ __align__(16) ulonglong2 sdata[kLanesMaxLen];  // (x, x), (y, y)
+  __shared__ LaneRef refs[kTpb / 32];
+  __shared__ ProposalSmem prop;
+  __shared__ int64_t run_sh;
+  __shared__ int last_sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  LaneRef& rf = refs[warp];
+  int cur = -1;  // instance whose data and proposal are staged
+  while (true) {
+    if (tid == 0) run_sh = (int64_t)atomicAdd(&hdr->tile_counter[1], 1u);
+    __syncthreads();
+    int64_t s = run_sh * run_tiles;
+    const int64_t s_end = s + run_tiles < n_tiles ? s + run_tiles : n_tiles;
+    if (s >= n_tiles) break;
+    while (s < s_end) {  // the same for the whole block
+      // the instance of slot s: the last with first <= s (32 probes a round)
+      int lo = 0, hi = n_inst;  // first[lo] <= s < first[hi]
+      while (hi - lo > 1) {
+        const int w = (hi - lo + 31) / 32, q = lo + lane * w;
+        const unsigned m = __ballot_sync(0xffffffffu, q < hi && __ldg(first + q) <= s);
+        const int f = 31 - __clz(m);  // lane 0 probes lo: m != 0
+        hi = min(hi, lo + (f + 1) * w);
+        lo += f * w;
+      }
+      const int b = lo;
+      const int64_t d0 = data_off[b], L = data_off[b + 1] - d0;
+      const int64_t N = part_off[b + 1] - part_off[b];
+      const int64_t tiles = (b + 1 < n_inst ? (int64_t)first[b + 1] : n_tiles) - first[b];
+      const int64_t t0 = s - first[b], t1 = min(tiles, s_end - first[b]);
+      __syncthreads();  // the previous run's data and refs have been read
+      if (b != cur) {
+        for (int l = tid; l < kLanesMaxLen && l < L; l += kTpb)
+          sdata[l] = make_ulonglong2(f2_pack(xs[d0 + l], xs[d0 + l]), f2_pack(ys[d0 + l], ys[d0 + l]));
+        if (LEARNED && warp == 0) load_proposal(p, proposal + (int64_t)b * 48, prop);
+        cur = b;
+      }
+      if (lane < kMaxDegrees) {
+        rf.arg[lane] = 0x7fffffff;
+#pragma unroll
+        for (int j = 0; j < kMaxCoef; ++j) rf.v[lane][j] = 0.0f;
+        rf.v[lane][6] = rf.v[lane][7] = -INFINITY;
       }
       __syncthreads();
-      if (warp == 0)
-        write_summary_warp(fin, fS, fS2, p.n_deg, p.min_deg, N,
-                           lane == 0 ? ld_volatile_i32(&hdr->status) : 0, out + b);
+      LaneSums a[kMaxDegrees];
+#pragma unroll
+      for (int k = 0; k < kMaxDegrees; ++k) lane_zero(a[k]);
+      int nan = 0;
+      const int64_t i_end = min(N, t1 * tile_traces);
+      // a warp takes 64 consecutive traces, two per lane
+      for (int64_t i0 = t0 * tile_traces + warp * 64; i0 < i_end; i0 += (kTpb / 32) * 64) {
+        float c[2][kMaxCoef], corr[2], lw[2];
+        int d[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int64_t i = i0 + u * 32 + lane;
+          const uint32_t gi = (uint32_t)(i < i_end ? i : 0);
+          const int n = LEARNED ? LearnedDraw{p, seed, (uint32_t)b, &prop}(gi, c[u], corr[u])
+                                : PriorDraw{p, seed, (uint32_t)b}(gi, c[u], corr[u]);
+          d[u] = i < i_end ? n - p.min_deg : -1;
+        }
+        {
+          unsigned long long cc[kMaxCoef];
+#pragma unroll
+          for (int k = 0; k < kMaxCoef; ++k) cc[k] = f2_pack(c[0][k], c[1][k]);
+          float ss[2] = {0.0f, 0.0f}, comp[2] = {0.0f, 0.0f};
+          unsigned long long part = 0ull;
+          auto point = [&](const ulonglong2 pt) {
+            unsigned long long f = cc[kMaxCoef - 1];
+#pragma unroll
+            for (int k = kMaxCoef - 2; k >= 0; --k) f = f2_fma(f, pt.x, cc[k]);
+            const unsigned long long r = f2_sub(pt.y, f);
+            part = f2_fma(r, r, part);
+          };
+          for (int64_t l = 0; l < L; l += 16) {  // blocks of 16 points, compensated between
+            const int nb = L - l < 16 ? (int)(L - l) : 16;
+            part = 0ull;
+            if (l >= kLanesMaxLen) {  // past what the plan announced
+              for (int j = 0; j < nb; ++j) {
+                const float xv = xs[d0 + l + j], yv = ys[d0 + l + j];
+                point(make_ulonglong2(f2_pack(xv, xv), f2_pack(yv, yv)));
+              }
+            } else if (nb == 16) {
+#pragma unroll 4
+              for (int j = 0; j < 16; ++j) point(sdata[l + j]);
+            } else {
+              for (int j = 0; j < nb; ++j) point(sdata[l + j]);
+            }
+            const float2 v = f2_unpack(part);
+            kahan_add(ss[0], comp[0], v.x);
+            kahan_add(ss[1], comp[1], v.y);
+          }
+#pragma unroll
+          for (int u = 0; u < 2; ++u) lw[u] = ss[u] * p.neg_half_inv_var + corr[u];
+        }
+        float4 f0[2], f1[2];
+        bool rare = false;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float4* rp = reinterpret_cast<const float4*>(rf.v[d[u] >= 0 ? d[u] : 0]);
+          f0[u] = rp[0];
+          f1[u] = rp[1];
+          rare |= d[u] >= 0 && !(lw[u] <= f1[u].w);  // a NaN too
+        }
+        if (__any_sync(0xffffffffu, rare)) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            nan |= d[u] >= 0 && lw[u] != lw[u];
+#pragma unroll
+            for (int k = 0; k < kMaxDegrees; ++k) {
+              const bool mine = d[u] == k && lw[u] > rf.v[k][7];
+              if (!__any_sync(0xffffffffu, mine)) continue;
+              const float mx = warp_max(mine ? lw[u] : -INFINITY);
+              // lanes hold increasing indices: the first lane at the maximum is the lowest
+              const int src = __ffs(__ballot_sync(0xffffffffu, mine && lw[u] == mx)) - 1;
+              const float m0 = rf.v[k][6];
+              if (!(mx <= m0 + kRebaseNats)) {
+                float g[kMaxCoef], nc[kMaxCoef];
+#pragma unroll
+                for (int j = 0; j < kMaxCoef; ++j) {
+                  nc[j] = __shfl_sync(0xffffffffu, c[u][j], src);
+                  g[j] = rf.v[k][j] - nc[j];
+                }
+                lane_move(a[k], g, m0 > -INFINITY ? expf(m0 - mx) : 0.0f);
+                __syncwarp();
+                if (lane == 0) {
+#pragma unroll
+                  for (int j = 0; j < kMaxCoef; ++j) rf.v[k][j] = nc[j];
+                  rf.v[k][6] = mx;
+                }
+              }
+              if (lane == src) {
+                rf.v[k][7] = mx;
+                rf.arg[k] = (int)(i0 + u * 32 + lane);
+              }
+              __syncwarp();
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float4* rp = reinterpret_cast<const float4*>(rf.v[d[u] >= 0 ? d[u] : 0]);
+            f0[u] = rp[0];
+            f1[u] = rp[1];
+          }
+        }
+        // under the prior few traces carry weight (FP32's exponential is 0 below -104)
+        if (!LEARNED) {
+          const bool some = !(lw[0] - f1[0].z < -104.0f) || !(lw[1] - f1[1].z < -104.0f);
+          if (!__any_sync(0xffffffffu, some)) continue;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          // -inf and NaN log-weights carry nothing
+          const float w = d[u] >= 0 && lw[u] > -INFINITY ? expf(lw[u] - f1[u].z) : 0.0f;
+          lane_add(a, d[u], w, c[u], f0[u], f1[u]);
+        }
+      }
+      // the warp's partials into the run's first slot, empty ones into the rest
+      DegPartial* slot0 = parts + (s * (kTpb / 32) + warp) * kMaxDegrees;
+#pragma unroll
+      for (int k = 0; k < kMaxDegrees; ++k) {
+        const DegPartial r = lane_partial(a[k], rf.v[k], rf.v[k][7], rf.arg[k]);
+        if (lane == 0) slot0[k] = r;
+      }
+      for (int64_t t = t0 + 1; t < t1; ++t)
+        if (lane < kMaxDegrees) deg_empty(slot0[(t - t0) * kWarpParts + lane]);
+      if (__any_sync(0xffffffffu, nan) && lane == 0) record_status(&hdr->status, PPL_ENAN);
+      // the last run of the instance merges its partials; the barrier and
+      // thread 0's fence order every warp's partial writes before the count
       __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        last_sh = atomicSub(&count[b], (int)(t1 - t0)) == (int)(t1 - t0);
+      }
+      __syncthreads();
+      if (last_sh) {
+        __threadfence();
+        finish_instance(p, parts + (int64_t)first[b] * kWarpParts, tiles, N, hdr, out + b);
+      }
+      s += t1 - t0;
     }
+    __syncthreads();  // run_sh is rewritten
   }
 }
 
 template <int PPT, bool LEARNED>
 static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const float* y,
                                     const int64_t* data_off, const int64_t* part_off,
-                                    int32_t n_inst, int64_t n_items, int blocks_per_sm,
+                                    int32_t n_inst, int64_t n_items, int64_t max_len, int64_t total, int blocks_per_sm,
                                     uint64_t seed, const float* proposal, char* ws,
                                     ppl_is_result* out, cudaStream_t s) {
   const BatchLayout l = batch_layout(n_items, n_inst);
@@ -186,6 +419,16 @@ static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const f
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(ws + l.inst_max, 0, (size_t)n_inst * kMaxDegrees * sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
+  if (max_len <= kLanesMaxLen && total >= kLanesMinTotal && total / n_inst >= kLanesMinMean) {
+    const int64_t blocks = (int64_t)num_sms() * 2;
+    const int run = (int)std::max<int64_t>(1, kRunTraces / (kTpb * PPT));
+    const int64_t runs = (n_items + run - 1) / run;
+    lanes_kernel<LEARNED><<<(unsigned)std::min(runs, blocks), kTpb, 0, s>>>(
+        p, x, y, data_off, part_off, n_inst, n_items, kTpb * PPT, run,
+        reinterpret_cast<const int32_t*>(ws + l.first), reinterpret_cast<int32_t*>(ws + l.count),
+        seed, proposal, hdr, reinterpret_cast<DegPartial*>(ws + l.parts), out);
+    return cudaGetLastError();
+  }
   const size_t smem = trace_smem_bytes<PPT>() + kBatchChunk * sizeof(float2);
   int unused = 0;
   e = device_once((const void*)batched_kernel<PPT, LEARNED>, &unused, [smem](int*) {
@@ -209,14 +452,15 @@ static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const f
 
 cudaError_t launch_batched(const PolyParams& p, const float* x, const float* y,
                            const int64_t* data_off, const int64_t* part_off, int32_t n_inst,
-                           int64_t n_items, int ppt, int blocks_per_sm, uint64_t seed,
+                           int64_t n_items, int64_t max_len, int64_t total, int ppt, int blocks_per_sm, uint64_t seed,
                            const float* proposal, char* ws, ppl_is_result* out, cudaStream_t s) {
 #define PPL_BATCHED_CASE(P)                                                                   \
   case P:                                                                                     \
-    return proposal ? launch_batched_t<P, true>(p, x, y, data_off, part_off, n_inst, n_items, \
+    return proposal ? launch_batched_t<P, true>(p, x, y, data_off, part_off, n_inst, n_items, max_len, total, \
                                                 blocks_per_sm, seed, proposal, ws, out, s)    \
                     : launch_batched_t<P, false>(p, x, y, data_off, part_off, n_inst,         \
-                                                 n_items, blocks_per_sm, seed, nullptr, ws,   \
+                                                 n_items, max_len, total, blocks_per_sm, seed, \
+                                                 nullptr, ws,                                 \
                                                  out, s);
   switch (ppt) {
     PPL_BATCHED_CASE(1)
@@ -369,7 +613,8 @@ ppl_status ppl_infer_is_batched(const ppl_model* model, const float* x, const fl
   if (plan->n_inst != n_inst || !valid_ppt(plan->ppt)) return PPL_EINVAL;
   if (ws_bytes < batch_layout(plan->n_items, n_inst).total) return PPL_EINVAL;
   const cudaError_t e =
-      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->ppt,
+      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len, plan->total_particles,
+                     plan->ppt,
                      plan->blocks_per_sm, seed, nullptr, static_cast<char*>(ws), out_dev,
                      (cudaStream_t)stream);
   return e == cudaSuccess ? PPL_OK : PPL_ECUDA;
@@ -390,7 +635,8 @@ ppl_status ppl_infer_is_learned(const ppl_model* model, const float* x, const fl
   if (plan->n_inst != n_inst || !valid_ppt(plan->ppt)) return PPL_EINVAL;
   if (ws_bytes < batch_layout(plan->n_items, n_inst).total) return PPL_EINVAL;
   const cudaError_t e =
-      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->ppt,
+      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len, plan->total_particles,
+                     plan->ppt,
                      plan->blocks_per_sm, seed, proposal, static_cast<char*>(ws), out_dev,
                      (cudaStream_t)stream);
   return e == cudaSuccess ? PPL_OK : PPL_ECUDA;

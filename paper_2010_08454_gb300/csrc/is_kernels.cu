@@ -8,6 +8,7 @@
 
 #include "dfloat.cuh"
 #include "kernels.h"
+#include "lanesums.cuh"
 #include "poly.cuh"
 #include "posterior.cuh"
 #include "stats.cuh"
@@ -413,7 +414,6 @@ constexpr int kPostPer = 4;                 // particles of a lane per tile
 constexpr int kPostU = 2;                   // of these in registers at once
 constexpr int kPostTile = 32 * kPostPer;    // particles of a warp's tile
 constexpr int kPostStages = 3;              // tiles in flight per warp
-constexpr float kRebaseNats = 8.0f;
 
 struct PostStage {
   float4 rec[kPostTile * 2];
@@ -474,26 +474,6 @@ __device__ __forceinline__ void post_fetch(PostStage* st, const ppl_poly_particl
   }
 }
 
-// A lane's sums of one degree as f32x2 pairs.
-struct PostSums {
-  unsigned long long s12, A[kMaxCoef / 2], B[kMaxCoef / 2];
-};
-
-// Move a lane's sums to a reference g below the old one (g = old - new per
-// coefficient), rescaling the weights by ex.
-__device__ __forceinline__ void post_move(PostSums& a, const float (&g)[kMaxCoef], float ex) {
-  const float2 s = f2_unpack(a.s12);
-  const unsigned long long ee = f2_pack(ex, ex), ss = f2_pack(s.x, s.x);
-#pragma unroll
-  for (int j = 0; j < kMaxCoef / 2; ++j) {
-    const unsigned long long gg = f2_pack(g[2 * j], g[2 * j + 1]);
-    const unsigned long long A1 = f2_fma(ss, gg, a.A[j]);  // A + S g
-    a.B[j] = f2_mul(ee, f2_fma(gg, f2_add(a.A[j], A1), a.B[j]));
-    a.A[j] = f2_mul(ee, A1);
-  }
-  a.s12 = f2_pack(s.x * ex, s.y * ex * ex);
-}
-
 __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
     PolyParams p, const ppl_poly_particle* __restrict__ rec, const float* __restrict__ lwin,
     int64_t N, WsHeader* hdr, DegPartial* parts, ppl_is_result* res) {
@@ -512,13 +492,9 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
     rf.arg[lane] = 0x7fffffff;
   }
   __syncthreads();
-  PostSums a[kMaxDegrees];
+  LaneSums a[kMaxDegrees];
 #pragma unroll
-  for (int k = 0; k < kMaxDegrees; ++k) {
-    a[k].s12 = 0ull;
-#pragma unroll
-    for (int j = 0; j < kMaxCoef / 2; ++j) a[k].A[j] = a[k].B[j] = 0ull;
-  }
+  for (int k = 0; k < kMaxDegrees; ++k) lane_zero(a[k]);
   int nan = 0, bad = 0;
   const int64_t tiles = (N + kPostTile - 1) / kPostTile;
   const int64_t step = (int64_t)gridDim.x * kPostWarps;
@@ -594,7 +570,7 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
               float g[kMaxCoef];
 #pragma unroll
               for (int j = 0; j < kMaxCoef; ++j) g[j] = rf.v[k][j] - cu[8 * src + j];
-              post_move(a[k], g, m0 > -INFINITY ? expf(m0 - mx) : 0.0f);
+              lane_move(a[k], g, m0 > -INFINITY ? expf(m0 - mx) : 0.0f);
               __syncwarp();
               if (lane < kMaxCoef) rf.v[k][lane] = cu[8 * src + lane];
               if (lane == 0) rf.v[k][6] = mx;
@@ -622,25 +598,8 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
       for (int u = 0; u < kPostU; ++u) {
         // -inf and NaN log-weights carry nothing
         const float w = lw[u] > -INFINITY ? expf(lw[u] - f1[u].z) : 0.0f;
-        const unsigned long long d2[kMaxCoef / 2] = {
-            f2_sub(f2_pack(r0[u].x, r0[u].y), f2_pack(f0[u].x, f0[u].y)),
-            f2_sub(f2_pack(r0[u].z, r0[u].w), f2_pack(f0[u].z, f0[u].w)),
-            f2_sub(f2_pack(r1[u].x, r1[u].y), f2_pack(f1[u].x, f1[u].y))};
-        unsigned long long q2[kMaxCoef / 2];
-#pragma unroll
-        for (int j = 0; j < kMaxCoef / 2; ++j) q2[j] = f2_mul(d2[j], d2[j]);
-        const unsigned long long one_w = f2_pack(1.0f, w);
-#pragma unroll
-        for (int k = 0; k < kMaxDegrees; ++k) {
-          const float wk = d[u] == k ? w : 0.0f;
-          const unsigned long long ww = f2_pack(wk, wk);
-          a[k].s12 = f2_fma(ww, one_w, a[k].s12);
-#pragma unroll
-          for (int j = 0; j < kMaxCoef / 2; ++j) {
-            a[k].A[j] = f2_fma(ww, d2[j], a[k].A[j]);
-            a[k].B[j] = f2_fma(ww, q2[j], a[k].B[j]);
-          }
-        }
+        const float c[kMaxCoef] = {r0[u].x, r0[u].y, r0[u].z, r0[u].w, r1[u].x, r1[u].y};
+        lane_add(a, d[u], w, c, f0[u], f1[u]);
       }
     }
     // after 1, 2, 4, .. tiles: the references move to the means
@@ -658,7 +617,7 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
           c[j] = r + warp_sum(j & 1 ? v.y : v.x) / S;
           g[j] = r - c[j];
         }
-        post_move(a[k], g, 1.0f);
+        lane_move(a[k], g, 1.0f);
         __syncwarp();
         if (lane == 0) {
 #pragma unroll
@@ -672,33 +631,8 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
   // the warp's partials: sums over its lanes, moved to the best trace's weight
 #pragma unroll
   for (int k = 0; k < kMaxDegrees; ++k) {
-    const float2 s = f2_unpack(a[k].s12);
-    const float S = warp_sum(s.x), S2 = warp_sum(s.y);
-    float A[kMaxCoef], B[kMaxCoef];
-#pragma unroll
-    for (int j = 0; j < kMaxCoef / 2; ++j) {
-      const float2 av = f2_unpack(a[k].A[j]), bv = f2_unpack(a[k].B[j]);
-      A[2 * j] = warp_sum(av.x);
-      A[2 * j + 1] = warp_sum(av.y);
-      B[2 * j] = warp_sum(bv.x);
-      B[2 * j + 1] = warp_sum(bv.y);
-    }
+    const DegPartial r = lane_partial(a[k], rf.v[k], rf.v[k][7], rf.arg[k]);
     if (lane == 0) {
-      DegPartial r;
-      deg_empty(r);
-      r.m = rf.v[k][7];
-      r.arg = rf.arg[k];
-      if (r.m > -INFINITY && S > 0.0f) {
-        const float ex = expf(rf.v[k][6] - r.m), inv = 1.0f / S;
-        r.S = S * ex;
-        r.S2 = S2 * ex * ex;
-#pragma unroll
-        for (int j = 0; j < kMaxCoef; ++j) {
-          const float sh = A[j] * inv;
-          r.mean[j] = rf.v[k][j] + sh;
-          r.M2[j] = fmaxf(fmaf(-sh, A[j], B[j]), 0.0f) * ex;
-        }
-      }
       wparts[warp][k] = r;
     }
   }

@@ -17,13 +17,15 @@ struct ProposalSmem {
   float cum[kMaxDegrees];
   float logq[kMaxDegrees];
   int base[kMaxDegrees];
-  float mu[kMaxSlots], s[kMaxSlots], logs[kMaxSlots], inv_s[kMaxSlots];
+  float4 slot[kMaxSlots];  // mu, s, 1 / s, log s: one load per coefficient
   float log_p, log_sigma, sigma, inv_sigma;
 };
 
-// Proposal of one data set from its 48 network outputs (one thread).
+// Proposal of one data set from its 48 network outputs, by the 32 lanes of one
+// warp: lane i takes slot i, every lane the degrees.
 __device__ __forceinline__ void load_proposal(const PolyParams& p, const float* o,
                                               ProposalSmem& ps) {
+  const int lane = threadIdx.x & 31;
   float mx = -INFINITY;
   for (int k = 0; k < p.n_deg; ++k) mx = fmaxf(mx, o[k]);
   float se = 0.0f;
@@ -32,28 +34,33 @@ __device__ __forceinline__ void load_proposal(const PolyParams& p, const float* 
   float cum = 0.0f;
   int base = 0;
   for (int k = 0; k < kMaxDegrees; ++k) {
+    float ck = 2.0f, lq = 0.0f;
+    int bk = 0;
     if (k < p.n_deg) {
       cum += expf(o[k] - mx) / se;
-      ps.cum[k] = cum;
-      ps.logq[k] = (o[k] - mx) - lse;
-      ps.base[k] = base;
+      ck = cum;
+      lq = (o[k] - mx) - lse;
+      bk = base;
       base += p.min_deg + k + p.coef_offset;
-    } else {
-      ps.cum[k] = 2.0f;
-      ps.logq[k] = 0.0f;
-      ps.base[k] = 0;
+    }
+    if (lane == 0) {
+      ps.cum[k] = ck;
+      ps.logq[k] = lq;
+      ps.base[k] = bk;
     }
   }
-  ps.sigma = p.prior_sigma;
-  ps.inv_sigma = 1.0f / p.prior_sigma;
-  ps.log_sigma = logf(p.prior_sigma);
-  ps.log_p = -logf((float)p.n_deg);
-  for (int i = 0; i < kMaxSlots && i < base; ++i) {
-    const float t = fminf(fmaxf(o[5 + 2 * i], -9.0f), 1.0f);
-    ps.mu[i] = p.prior_sigma * o[4 + 2 * i];
-    ps.s[i] = p.prior_sigma * expf(t);
-    ps.inv_s[i] = 1.0f / ps.s[i];  // (the prior's reciprocal when s equals sigma)
-    ps.logs[i] = ps.log_sigma + t;
+  const float log_sigma = logf(p.prior_sigma);
+  if (lane == 0) {
+    ps.sigma = p.prior_sigma;
+    ps.inv_sigma = 1.0f / p.prior_sigma;
+    ps.log_sigma = log_sigma;
+    ps.log_p = -logf((float)p.n_deg);
+  }
+  if (lane < kMaxSlots && lane < base) {
+    const float t = fminf(fmaxf(o[5 + 2 * lane], -9.0f), 1.0f);
+    const float s = p.prior_sigma * expf(t);
+    // (1 / s is the prior's reciprocal when s equals sigma)
+    ps.slot[lane] = make_float4(p.prior_sigma * o[4 + 2 * lane], s, 1.0f / s, log_sigma + t);
   }
 }
 
@@ -88,10 +95,10 @@ struct LearnedDraw {
 #pragma unroll
     for (int j = 0; j < kMaxCoef; ++j) {
       if (j < ncoef) {
-        const float mu = ps->mu[base + j], s = ps->s[base + j];
-        c[j] = fmaf(s, z[j], mu);
+        const float4 q = ps->slot[base + j];
+        c[j] = fmaf(q.y, z[j], q.x);
         cr += log_normal32(c[j], 0.0f, ps->inv_sigma, ps->log_sigma) -
-              log_normal32(c[j], mu, ps->inv_s[base + j], ps->logs[base + j]);
+              log_normal32(c[j], q.x, q.z, q.w);
       } else {
         c[j] = 0.0f;
       }
