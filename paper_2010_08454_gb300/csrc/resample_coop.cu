@@ -24,9 +24,9 @@
 //      A chunk that lies wholly inside one block's run and has at most two
 //      outputs per particle (near-uniform weights) is written instead in the
 //      scatter form of the same definition: particle j's offspring are the
-//      outputs [K(C_{j-1}), K(C_j)), K(c) = #{k : u + k stride < c}; the
-//      block writes the chunk's ancestors into a table in shared memory,
-//      then the ancestors and the records output by output.
+//      outputs [K(C_{j-1}), K(C_j)), K(c) = #{k : u + k stride < c}; each
+//      particle marks the first of them in a table in shared memory, and the
+//      warps resolve the marks and copy the records a row of outputs at a time.
 //
 // Every item costs at most 4096 weights and 256 outputs whatever the weights
 // are: a chunk holding most of the mass (degenerate importance weights)
@@ -54,7 +54,6 @@ constexpr int kRcBatch = 32;                          // chunks summed between b
 // items over the blocks, so that a block whose run crosses many sparsely
 // used chunks takes correspondingly fewer items.
 constexpr int kRcPrefixCost = 128;
-constexpr int kRcShort = 4;      // offspring a lane writes alone in the scatter form
 constexpr int kRcScatterOut = 2 * (int)kRcChunk;  // outputs of a chunk written in the scatter form
 constexpr int kRcJobBlk = 8;     // chunk totals the layout job's first pass loads at once per thread
 constexpr int kRcJobPer = 4;     // chunks per thread in a tile of the layout job
@@ -89,12 +88,12 @@ struct RcArgs {
   int64_t* kfirst;  // [n_chunks + 1] first output of each chunk (K_c), K_last = m
   int64_t* ioff;    // [n_chunks + 1] first work item of each chunk
   // fused gather (rec_words > 0): rec_out[k] = rec_in[a_k], records of
-  // rec_words words of 16 bytes (or of 4 bytes when rec_word4), rec_in
+  // rec_words words of 16 bytes (or of 4 bytes: RecKind), rec_in
   // holding the n particles' records
   const void* rec_in;
   void* rec_out;
   int32_t rec_words;
-  int32_t rec_word4;
+  uint32_t rec_inv;    // ceil(2^32 / rec_words), rec_words > 1
   // one shard of a population split over devices (planned != 0): the
   // weights are quantised for a population of n_scale particles, the layout
   // (stride, u) and this shard's exclusive prefix c_base are given, its
@@ -105,6 +104,10 @@ struct RcArgs {
   uint64_t p_stride, p_u, c_base;
   int64_t k_off, k_end, j_off;
 };
+
+// REC: what the fused gather copies (one instantiation each: the kernel is held
+// to 64 registers, and the copies it does not make would cost it spills).
+enum RecKind { kRecNone = 0, kRec32 = 1, kRecWords16 = 2, kRecWords4 = 3 };
 
 // The records of outputs k0 .. k0 + nB - 1 of an item, by one warp: output j
 // copies the record of ancestor anc_of(j); consecutive lanes take consecutive
@@ -127,53 +130,59 @@ __device__ __forceinline__ void gather_words(const V* in, V* out_all, int W, int
   }
 }
 
-template <class AncOf>
+template <int REC, class AncOf>
 __device__ __forceinline__ void gather_item(const RcArgs& a, int64_t k0, int nB, AncOf anc_of,
                                             int lane) {
-  if (a.rec_word4)
+  if constexpr (REC == kRecWords4)
     gather_words(reinterpret_cast<const uint32_t*>(a.rec_in), reinterpret_cast<uint32_t*>(a.rec_out),
                  a.rec_words, k0, nB, anc_of, lane);
-  else
+  else if constexpr (REC != kRecNone)
     gather_words(reinterpret_cast<const uint4*>(a.rec_in), reinterpret_cast<uint4*>(a.rec_out),
                  a.rec_words, k0, nB, anc_of, lane);
 }
 
-// The records of outputs k0 .. k0 + n - 1 by the whole block, from the
-// ancestors in shared memory: thread t copies words t, t + kRcTpb, .., four
-// loads in flight before their stores (coalesced on both sides, the
-// ancestors being non-decreasing).
-template <typename V>
-__device__ __forceinline__ void gather_block_words(const V* __restrict__ in, V* __restrict__ out,
-                                                   int W, int64_t k0, int n, const int32_t* sOut,
-                                                   int tid) {
-  const int total = n * W;
-  out += k0 * W;
-  for (int e0 = tid; e0 < total; e0 += 4 * kRcTpb) {
-    V v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = e0 + q * kRcTpb;
-      if (e < total) {
-        const int j = e / W;
-        v[q] = in[(int64_t)sOut[j] * W + (e - j * W)];
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int e = e0 + q * kRcTpb;
-      if (e < total) out[e] = v[q];
-    }
-  }
+// One 32-byte record in one access (sm_100 and later; 32-byte aligned).
+struct Rec32 {
+  float v[8];
+};
+__device__ __forceinline__ Rec32 ld_rec32(const void* p) {
+  Rec32 r;
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]),
+                 "=f"(r.v[6]), "=f"(r.v[7])
+               : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void st_rec32(void* p, const Rec32& r) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r.v[0]),
+               "f"(r.v[1]), "f"(r.v[2]), "f"(r.v[3]), "f"(r.v[4]), "f"(r.v[5]), "f"(r.v[6]),
+               "f"(r.v[7])
+               : "memory");
 }
 
-__device__ __forceinline__ void gather_block(const RcArgs& a, int64_t k0, int n,
-                                             const int32_t* sOut, int tid) {
-  if (a.rec_word4)
-    gather_block_words(reinterpret_cast<const uint32_t*>(a.rec_in),
-                       reinterpret_cast<uint32_t*>(a.rec_out), a.rec_words, k0, n, sOut, tid);
-  else
-    gather_block_words(reinterpret_cast<const uint4*>(a.rec_in), reinterpret_cast<uint4*>(a.rec_out),
-                       a.rec_words, k0, n, sOut, tid);
+// The records of one row of a scattered chunk (n <= 32 consecutive outputs from
+// k0, lane l's ancestor an), W words each: consecutive lanes take consecutive
+// words, up to four loads in flight before their stores.
+template <typename V>
+__device__ __forceinline__ void gather_row(const V* __restrict__ in, V* __restrict__ out, int W,
+                                           uint32_t inv_w, int64_t k0, int n, int an, int lane) {
+  constexpr int kU = sizeof(V) == 4 ? 4 : 2;
+  out += k0 * W;
+  for (int w0 = 0; w0 < W; w0 += kU) {
+    V v[kU];
+#pragma unroll
+    for (int i = 0; i < kU; ++i) {
+      const int e = (w0 + i) * 32 + lane;
+      const int j = W > 1 ? (int)__umulhi((uint32_t)e, inv_w) : e;  // e / W, e < 2^13
+      const int src = __shfl_sync(0xffffffffu, an, j & 31);
+      if (w0 + i < W && j < n) v[i] = in[(int64_t)src * W + (e - j * W)];
+    }
+#pragma unroll
+    for (int i = 0; i < kU; ++i) {
+      const int e = (w0 + i) * 32 + lane;
+      if (w0 + i < W && e < n * W) out[e] = v[i];
+    }
+  }
 }
 
 // The weights of one thread's kRcItems particles from `base`: FP32
@@ -330,14 +339,14 @@ __device__ __forceinline__ void seg_lookup(const RcArgs& a, int64_t it, int64_t 
   if (lane < 6) out[lane] = v;
 }
 
-template <bool FROM_LW>
+template <bool FROM_LW, int REC>
 __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
   if (a.gate && *a.gate == 0) return;  // every block reads the same flag
   extern __shared__ __align__(16) unsigned char rc_dyn[];
   uint64_t* sA = reinterpret_cast<uint64_t*>(rc_dyn);  // [kRcChunk] prefix sums of a chunk
   uint64_t* sL2 = sA + kRcChunk;                        // [kRcTpb] every 8th of them
   int32_t* sW = reinterpret_cast<int32_t*>(sL2 + kRcTpb);  // [warp][kRcItemOut] ancestors
-  int32_t* sOut = sW + kRcWarps * kRcItemOut;  // [kRcScatterOut] a scattered chunk's ancestors
+  int32_t* marks = sW + kRcWarps * kRcItemOut;  // [kRcScatterOut] a scattered chunk's marks, 0 between
   __shared__ uint64_t sL1[kRcChunk / 256];  // every 256th prefix sum
   static_assert(3 * kRcJobTile * 8 <= kRcChunk * 8 + kRcTpb * 8 + kRcWarps * kRcItemOut * 4,
                 "the layout job's tile tables fit in the dynamic shared memory");
@@ -348,6 +357,7 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
   __shared__ int64_t seg_sh[2][6];  // chunk, its first and end unit, first and end output, C at its start
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned G = gridDim.x;
+  bool cleared = false;  // the marks, before the block's first scattered chunk
   float m_lw = 0.0f, scale = 0.0f;
   if (FROM_LW) {
     m_lw = a.known_max ? (float)*a.known_max : a.hdr->max_lw;
@@ -570,8 +580,8 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
     // particle on average, is written in the scatter form (below)
     const int nCw = (int)(a.n - cb < kRcChunk ? a.n - cb : kRcChunk);
     const bool scatter = it <= io0 && seg_sh[cur][2] <= it1 && kn - kc <= kRcScatterOut;
-    if (xs < io1) {  // the same for every thread of the block: the chunk's inclusive
-      // prefix sums, every 8th and every 256th
+    const bool write = xs < io1;  // the same for every thread of the block
+    if (write) {  // the chunk's inclusive prefix sums
       uint64_t p[kRcItems];
       load_weights<FROM_LW>(a, cb + (int64_t)tid * kRcItems, m_lw, scale, p, bad);
 #pragma unroll
@@ -579,56 +589,73 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
       const uint64_t own = p[kRcItems - 1];
       const uint64_t inc = warp_scan_acc<FROM_LW>(own, lane);
       if (lane == 31) wtot[warp] = inc;
+      if (scatter && !cleared) {
+        for (int i = tid; i < kRcScatterOut; i += kRcTpb) marks[i] = 0;
+        cleared = true;
+      }
       __syncthreads();
       const uint64_t v = lane < kRcWarps ? wtot[lane] : 0ull;
       const uint64_t wi = warp_scan_acc<FROM_LW>(v, lane);
       const uint64_t base = acc_add<FROM_LW>(
           cstart, acc_add<FROM_LW>(__shfl_sync(0xffffffffu, wi - v, warp), inc - own));
+      if (scatter) {
+        // the scatter form of the same definition: particle j's offspring are
+        // the outputs k with C_{j-1} <= u + k stride < C_j, i.e. [K(C_{j-1}),
+        // K(C_j)) with K(c) = positions below c.  A thread walks its eight
+        // particles and marks, in the chunk's output table, each one's first
+        // offspring and the first output of every later row of 32 that its
+        // offspring reach: a slot's ancestor is then the last mark at or
+        // before it in its own row.
+        const int n_out = (int)(kn - kc);
+        const StepDiv dv(u + (uint64_t)kc * stride, stride);
+        int k0 = min(dv.below(base), n_out);
 #pragma unroll
-      for (int r = 0; r < kRcItems; ++r) sA[tid * kRcItems + r] = acc_add<FROM_LW>(base, p[r]);
-      const uint64_t last = acc_add<FROM_LW>(base, own);
-      sL2[tid] = last;
-      if ((tid & 31) == 31) sL1[tid >> 5] = last;  // thread 32 i + 31 ends 256-block i
+        for (int r = 0; r < kRcItems; ++r) {
+          const int k1 = min(dv.below(acc_add<FROM_LW>(base, p[r])), n_out);
+          if (k1 > k0) {
+            const int32_t mark = (int32_t)(tid * kRcItems + r) + 1;
+            marks[k0] = mark;
+            for (int row = k0 / 32 + 1; row * 32 < k1; ++row) marks[row * 32] = mark;
+          }
+          k0 = k1;
+        }
+      } else {  // every sum, every 8th and every 256th for the merge path
+#pragma unroll
+        for (int r = 0; r < kRcItems; ++r) sA[tid * kRcItems + r] = acc_add<FROM_LW>(base, p[r]);
+        const uint64_t last = acc_add<FROM_LW>(base, own);
+        sL2[tid] = last;
+        if ((tid & 31) == 31) sL1[tid >> 5] = last;  // thread 32 i + 31 ends 256-block i
+      }
       __syncthreads();
     }
     // warp 0 fetches the next chunk's descriptor while the others take this
     // chunk's items
     if (more && warp == 0) seg_lookup(a, io1, ch + 1, seg_sh[cur ^ 1], lane);
-    if (xs < io1 && scatter) {
-      // the scatter form of the same definition: particle j's offspring are
-      // the outputs k with C_{j-1} <= u + k stride < C_j, i.e. [K(C_{j-1}),
-      // K(C_j)) with K(c) = positions below c.  Lane l of a warp takes
-      // particle 32 w + l of each 512-particle slice and writes its
-      // ancestor index into the chunk's output table in shared memory (a
-      // particle with more than kRcShort offspring by its whole warp); the
-      // block then writes the ancestors and gathers the records output by
-      // output, several loads in flight per thread.
-      const int n_out = (int)(kn - kc);
-      for (int j0 = 0; j0 < nCw; j0 += kRcTpb) {
-        const int j = j0 + tid;  // the same slice for the whole warp
-        const bool has = j < nCw;
-        const int64_t ke = has ? positions_below_inv(sA[j], u, sv, a.m) : a.m;
-        int64_t ks = __shfl_up_sync(0xffffffffu, ke, 1);
-        if (lane == 0)
-          ks = has ? positions_below_inv(j == 0 ? cstart : sA[j - 1], u, sv, a.m) : a.m;
-        const int32_t an = (int32_t)(cb + j);
-        const bool longr = has && ke - ks > kRcShort;
-        if (has && !longr)
-          for (int64_t k = ks; k < ke; ++k) sOut[k - kc] = an;
-        unsigned lm = __ballot_sync(0xffffffffu, longr);
-        while (lm) {
-          const int src = __ffs(lm) - 1;
-          lm &= lm - 1;
-          const int s0 = (int)(__shfl_sync(0xffffffffu, ks, src) - kc);
-          const int s1 = (int)(__shfl_sync(0xffffffffu, ke, src) - kc);
-          const int32_t as = __shfl_sync(0xffffffffu, an, src);
-          for (int k = s0 + lane; k < s1; k += 32) sOut[k] = as;
+    if (write && scatter) {
+      const int n_out = (int)(kn - kc), n_rows = (n_out + 31) / 32;
+      // (one row at a time: two or four together spill at 64 registers, 457 and
+      // 549 us against 439 for a summary and this call on 2^24 records)
+      for (int row = warp; row < n_rows; row += kRcWarps) {
+        const int j0 = row * 32, n = min(32, n_out - j0);
+        const int64_t k0 = kc - a.k_off + j0;
+        const int32_t mk = marks[j0 + lane];
+        marks[j0 + lane] = 0;
+        const unsigned at = __ballot_sync(0xffffffffu, mk != 0) & (0xffffffffu >> (31 - lane));
+        const int an = (int)cb + __shfl_sync(0xffffffffu, mk, 31 - __clz(at)) - 1;
+        if (lane < n) a.anc[k0 + lane] = an + (int32_t)a.j_off;
+        if constexpr (REC == kRec32) {
+          if (lane < n)
+            st_rec32(static_cast<char*>(a.rec_out) + (k0 + lane) * 32,
+                     ld_rec32(static_cast<const char*>(a.rec_in) + (int64_t)an * 32));
+        } else if constexpr (REC == kRecWords16) {
+          gather_row(static_cast<const uint4*>(a.rec_in), static_cast<uint4*>(a.rec_out),
+                     a.rec_words, a.rec_inv, k0, n, an, lane);
+        } else if constexpr (REC == kRecWords4) {
+          gather_row(static_cast<const uint32_t*>(a.rec_in), static_cast<uint32_t*>(a.rec_out),
+                     a.rec_words, a.rec_inv, k0, n, an, lane);
         }
       }
-      __syncthreads();
-      for (int e = tid; e < n_out; e += kRcTpb) a.anc[kc - a.k_off + e] = sOut[e] + (int32_t)a.j_off;
-      if (a.rec_words > 0) gather_block(a, kc - a.k_off, n_out, sOut, tid);
-    } else if (xs < io1 && !(more && warp == 0)) {
+    } else if (write && !(more && warp == 0)) {
       const int nC = (int)(a.n - cb < kRcChunk ? a.n - cb : kRcChunk);
       const int w0 = more ? 1 : 0, nw = kRcWarps - w0;
       for (int64_t x = xs + (warp - w0); x < io1; x += nw) {
@@ -642,8 +669,7 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         if (posl < sA[ia]) {  // one ancestor for the whole item (degenerate weights)
           const int32_t an = (int32_t)(cb + ia);
           for (int jj = lane; jj < nB; jj += 32) a.anc[k0 - a.k_off + jj] = an + (int32_t)a.j_off;
-          if (a.rec_words > 0)
-            gather_item(a, k0 - a.k_off, nB, [an](int) { return an; }, lane);
+          gather_item<REC>(a, k0 - a.k_off, nB, [an](int) { return an; }, lane);
           continue;
         }
         const int ib = min(chunk_first_above(sA, sL2, sL1, posl, lane) + 1, nC);
@@ -672,8 +698,7 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         }
         __syncwarp();
         for (int jj = lane; jj < nB; jj += 32) a.anc[k0 - a.k_off + jj] = sWw[jj] + (int32_t)a.j_off;
-        if (a.rec_words > 0)
-          gather_item(a, k0 - a.k_off, nB, [sWw](int j) { return sWw[j]; }, lane);
+        gather_item<REC>(a, k0 - a.k_off, nB, [sWw](int j) { return sWw[j]; }, lane);
         __syncwarp();  // sWw is rewritten by the warp's next item
       }
     }
@@ -764,14 +789,16 @@ cudaError_t launch_resample_coop(const float* lw, const uint64_t* q_fixed, const
   a.rec_in = rec_in;
   a.rec_out = rec_out;
   a.rec_words = 0;
-  a.rec_word4 = 0;
+  a.rec_inv = 0;
+  int rec = kRecNone;
   if (rec_in) {
     const uintptr_t al = reinterpret_cast<uintptr_t>(rec_in) | reinterpret_cast<uintptr_t>(rec_out);
     if (!rec_out || rec_bytes <= 0 || rec_bytes > 1024 || rec_bytes % 4 || (al & 3))
       return cudaErrorInvalidValue;
     const bool w16 = rec_bytes % 16 == 0 && (al & 15) == 0;
-    a.rec_word4 = w16 ? 0 : 1;
     a.rec_words = (int32_t)(w16 ? rec_bytes / 16 : rec_bytes / 4);
+    rec = rec_bytes == 32 && (al & 31) == 0 ? kRec32 : (w16 ? kRecWords16 : kRecWords4);
+    a.rec_inv = a.rec_words > 1 ? (uint32_t)((((uint64_t)1 << 32) + a.rec_words - 1) / a.rec_words) : 0;
   }
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -786,7 +813,12 @@ cudaError_t launch_resample_coop(const float* lw, const uint64_t* q_fixed, const
   constexpr size_t dyn = (size_t)kRcChunk * sizeof(uint64_t) + (size_t)kRcTpb * sizeof(uint64_t) +
                          (size_t)kRcWarps * kRcItemOut * sizeof(int32_t) +
                          (size_t)kRcScatterOut * sizeof(int32_t);
-  const void* fn = lw ? (const void*)resample_coop_kernel<true> : (const void*)resample_coop_kernel<false>;
+  if (!lw && rec != kRecNone) return cudaErrorInvalidValue;  // records go with log-weights
+  const void* fn = !lw                  ? (const void*)resample_coop_kernel<false, kRecNone>
+                   : rec == kRecNone    ? (const void*)resample_coop_kernel<true, kRecNone>
+                   : rec == kRec32      ? (const void*)resample_coop_kernel<true, kRec32>
+                   : rec == kRecWords16 ? (const void*)resample_coop_kernel<true, kRecWords16>
+                                        : (const void*)resample_coop_kernel<true, kRecWords4>;
   // once per kernel and device: the shared-memory attribute and the residency
   int per_sm = 0;
   const cudaError_t e = device_once(fn, &per_sm, [fn](int* v) {

@@ -46,30 +46,6 @@ struct __align__(16) SmcPart {
   int nan;
 };
 
-// Division of the resampling positions by their stride when the quotient is
-// small: k(c) = #{j >= 0 : pos0 + j stride < c} for c - pos0 <= 2^16 stride
-// (more outputs than a block's table or a cluster holds).
-// With the stride's leading 16 bits the quotient's FP32 estimate is within
-// one of the exact one, and one remainder settles it: 15 instructions where
-// the general division of two 64-bit integers takes about 50.
-struct StepDiv {
-  uint64_t pos0, stride;
-  float inv;
-  int sh;
-  __device__ __forceinline__ StepDiv(uint64_t p, uint64_t s) : pos0(p), stride(s) {
-    sh = max(0, 48 - __clzll(s));  // s >> sh < 2^16
-    inv = __frcp_rn(lead_f32(s) * __int_as_float((127 - sh) << 23));
-  }
-  __device__ __forceinline__ int below(uint64_t c) const {
-    if (c <= pos0) return 0;
-    const uint64_t num = c - pos0 - 1;
-    int64_t q = (int64_t)__float2uint_rz(__uint2float_rz((uint32_t)(num >> sh)) * inv);
-    const int64_t r = (int64_t)(num - (uint64_t)q * stride);
-    q += r < 0 ? -1 : (r >= (int64_t)stride ? 1 : 0);
-    return (int)q + 1;
-  }
-};
-
 // What one step leaves for the evidence and ESS outputs, which are formed in
 // FP64 once after the last step: M the maximum log-weight, S and S2 the sums of
 // exp(lw - M) and exp(2 (lw - M)) as unevaluated FP32 pairs.
