@@ -829,12 +829,7 @@ cudaError_t launch_resample_coop(const float* lw, const uint64_t* q_fixed, const
     return r;
   });
   if (e != cudaSuccess) return e;
-  // every resident block, but not many more than have something to do (two per
-  // chunk, or a few items each): the grid barrier costs by the block
-  const int64_t outputs = shard ? shard->k_end - shard->k_first : m;
-  const int64_t grid = std::min<int64_t>(
-      (int64_t)num_sms() * per_sm,
-      std::max<int64_t>(2 * a.n_chunks, outputs / (8 * kRcItemOut) + 1));
+  const int64_t grid = (int64_t)num_sms() * per_sm;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kRcTpb), args, dyn, s);
 }
