@@ -53,7 +53,7 @@ MEASURED_TRAFFIC = {
     "resample_coop_kernel": {"bytes": 67495680 + 539461888,
                              "sources": ["resample_coop.cu", "gridsync.cuh", "fixedpoint.cuh",
                                          "rng.cuh", "kernels.h", "common.cuh"],
-                             "sha256": "ad58fbb3e79d1203"},
+                             "sha256": "1b0e565ae02a899d"},
 }
 
 

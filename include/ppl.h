@@ -384,9 +384,10 @@ ppl_status ppl_smc_step(const ppl_model* model, float y_t, int32_t t, uint64_t s
                         double* logz_est, void* ws, size_t ws_bytes, ppl_stream stream);
 
 /* The whole bootstrap filter of ppl_smc_step for t = 1..T in one persistent
- * cooperative kernel: x_0 = 0, lw_0 = 0, observations y [dev, FP32, T]; the
- * particles stay in registers between steps, which are separated by bounded
- * grid barriers.  Each step computes exactly what ppl_smc_step computes.
+ * kernel: x_0 = 0, lw_0 = 0, observations y [dev, FP32, T]; the particles stay
+ * in registers between steps, which are separated by bounded grid barriers
+ * (up to 32768 particles: by the barriers of one thread-block cluster, the
+ * same results).  Each step computes exactly what ppl_smc_step computes.
  * Writes x_out, lw_out [dev, n] (the final population), *logz_out [dev, FP64]
  * (the evidence estimate), resampled_out [dev, int32, T] and ess_out [dev,
  * FP64, T] (ESS before resampling).  n must fit the resident threads, at

@@ -9,7 +9,8 @@
 // launch itself only clears counters and starts one kernel, so it can be
 // captured in a CUDA graph and replayed.  The autotuner picks the traces per
 // thread and the resident blocks per SM by timing the candidates, and caches
-// the choice in a JSON file.
+// the choice in a JSON file.  Large batches of short data sets run in a kernel
+// of their own (lanes_kernel).
 #include <stdio.h>
 #include <string.h>
 
@@ -613,8 +614,8 @@ ppl_status ppl_infer_is_batched(const ppl_model* model, const float* x, const fl
   if (plan->n_inst != n_inst || !valid_ppt(plan->ppt)) return PPL_EINVAL;
   if (ws_bytes < batch_layout(plan->n_items, n_inst).total) return PPL_EINVAL;
   const cudaError_t e =
-      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len, plan->total_particles,
-                     plan->ppt,
+      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len,
+                     plan->total_particles, plan->ppt,
                      plan->blocks_per_sm, seed, nullptr, static_cast<char*>(ws), out_dev,
                      (cudaStream_t)stream);
   return e == cudaSuccess ? PPL_OK : PPL_ECUDA;
@@ -635,8 +636,8 @@ ppl_status ppl_infer_is_learned(const ppl_model* model, const float* x, const fl
   if (plan->n_inst != n_inst || !valid_ppt(plan->ppt)) return PPL_EINVAL;
   if (ws_bytes < batch_layout(plan->n_items, n_inst).total) return PPL_EINVAL;
   const cudaError_t e =
-      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len, plan->total_particles,
-                     plan->ppt,
+      launch_batched(p, x, y, data_off, part_off, n_inst, plan->n_items, plan->max_len,
+                     plan->total_particles, plan->ppt,
                      plan->blocks_per_sm, seed, proposal, static_cast<char*>(ws), out_dev,
                      (cudaStream_t)stream);
   return e == cudaSuccess ? PPL_OK : PPL_ECUDA;

@@ -1,6 +1,7 @@
 // The whole bootstrap particle filter on the linear-Gaussian state-space model
-// in one persistent, cooperative kernel (particle methods: the paper's stated
-// future work, §6; observe as in §3.4, Fig. 2).  One block of 1024 threads per
+// in one persistent kernel (particle methods: the paper's stated future work,
+// §6; observe as in §3.4, Fig. 2): a cooperative grid, described here, or for
+// small populations one thread-block cluster (smc_cluster_kernel).  One block of 1024 threads per
 // SM; each thread keeps its R particles' state and log-weights in registers
 // for all T steps; the steps are separated by grid barriers instead of kernel
 // launches.  The arithmetic of a step is exactly that of ppl_smc_step (same
