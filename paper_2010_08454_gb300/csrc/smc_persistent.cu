@@ -123,8 +123,6 @@ __device__ __forceinline__ void smc_outputs(const SmcArgs& a, double* sh_z) {
   }
 }
 
-// Thread `tid` of block b holds particles i0 .. i0 + R - 1, i0 = (b kSmcTpb + tid) R,
-// so a thread's fixed-point weights are consecutive terms of the prefix sum.
 // Inclusive warp scan.  The filter's weights are quantised log-weights, whose
 // sums cannot pass 2^61 (N weights of at most 2^(61 - ceil(log2 N))): plain sums.
 __device__ __forceinline__ uint64_t warp_scan_plain(uint64_t v, int lane) {
@@ -136,6 +134,8 @@ __device__ __forceinline__ uint64_t warp_scan_plain(uint64_t v, int lane) {
   return v;
 }
 
+// Thread `tid` of block b holds particles i0 .. i0 + R - 1, i0 = (b kSmcTpb + tid) R,
+// so a thread's fixed-point weights are consecutive terms of the prefix sum.
 template <int R>
 __global__ void __launch_bounds__(kSmcTpb, 1) smc_persistent_kernel(SmcArgs a) {
   constexpr int64_t P = (int64_t)kSmcTpb * R;  // particles of one block
