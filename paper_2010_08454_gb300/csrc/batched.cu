@@ -70,16 +70,8 @@ __device__ __forceinline__ void finish_instance(const PolyParams& p, const DegPa
   __shared__ DegPartial fin[kMaxDegrees];
   __shared__ float2 fS[kMaxDegrees], fS2[kMaxDegrees];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (warp < kMaxDegrees) {  // (tile, warp) partials of degree `warp`
-    DegPartial a;
-    DegSums ds;
-    merge_degree(parts, (int)(tiles * (kTpb / 32)), warp, lane, a, ds);
-    if (lane == 0) {
-      fin[warp] = a;
-      fS[warp] = ds.S;
-      fS2[warp] = ds.S2;
-    }
-  }
+  if (warp < kMaxDegrees)  // (tile, warp) partials of degree `warp`
+    merge_degree(parts, (int)(tiles * (kTpb / 32)), warp, lane, fin + warp, fS + warp, fS2 + warp);
   __syncthreads();
   if (warp == 0)
     write_summary_warp(fin, fS, fS2, p.n_deg, p.min_deg, N,

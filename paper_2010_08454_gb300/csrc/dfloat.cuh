@@ -19,6 +19,11 @@ __device__ __forceinline__ float2 df_add(float2 a, float2 b) {
   const float hi = __fadd_rn(s, t);
   return make_float2(hi, __fsub_rn(t, __fsub_rn(hi, s)));
 }
+// a + b of two FP32 numbers, exactly.
+__device__ __forceinline__ float2 df_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
 __device__ __forceinline__ float2 df_neg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 df_prod(float a, float b) {
   const float p = __fmul_rn(a, b);
@@ -35,6 +40,9 @@ __device__ __forceinline__ float2 df_mul(float2 a, float b) {
 }
 __device__ __forceinline__ float2 df_shfl_xor(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ float2 df_shfl(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 __device__ __forceinline__ float2 df_warp_sum(float2 v) {
 #pragma unroll
@@ -98,5 +106,47 @@ __device__ __forceinline__ ExpSplit exp_split(float d) {
 
 // 2^n as an FP32 value, for n in [-126, 127].
 __device__ __forceinline__ float exp2i(int n) { return __int_as_float((127 + n) << 23); }
+
+// Paired FP32 arithmetic (PTX f32x2, sm_100 and later): two lanes of IEEE
+// single precision in one 64-bit register, each half rounded exactly as the
+// scalar instruction would round it.  One instruction does the work of two.
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return make_float2(lo, hi);
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// The products in two scalar instructions: ptxas may fuse a f32x2 multiplication
+// into the f32x2 additions of its result, and then no rounded product exists.
+__device__ __forceinline__ unsigned long long f2_mul_rn(unsigned long long a, unsigned long long b) {
+  const float2 x = f2_unpack(a), y = f2_unpack(b);
+  return f2_pack(__fmul_rn(x.x, y.x), __fmul_rn(x.y, y.y));
+}
 
 }  // namespace ppl

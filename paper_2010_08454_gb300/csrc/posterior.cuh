@@ -151,7 +151,7 @@ __device__ __forceinline__ void write_summary_warp(const DegPartial* p, const fl
     const int kk = lane / kMaxCoef, j = lane % kMaxCoef;
     const bool ok = kk < n_deg && p[kk].m != -INFINITY && S[kk].x > 0.0f && p[kk].S > 0.0f;
     res->deg_mean[kk][j] = ok ? (double)p[kk].mean[j] : 0.0;
-    res->deg_var[kk][j] = ok ? (double)__fdiv_rn(p[kk].M2[j], p[kk].S) : 0.0;
+    res->deg_var[kk][j] = ok ? (double)df_div(make_float2(p[kk].M2[j], 0.0f), S[kk]) : 0.0;
   }
   // pooled coefficient means (written by lanes 0-5) and the heaviest degree
   {
@@ -229,27 +229,69 @@ struct DegSums {
 // Final merge of the per-block partials, by the last block: warp k merges
 // degree k's partials (merge_degree), warp 0 writes the summary.
 // ---------------------------------------------------------------------------
-// Warp `warp` (< kMaxDegrees) merges degree `warp` of G block partials in two
-// passes over them: the maximum and its index first, then every partial's
-// sums rescaled to that maximum once and added (S, S2 and sum w (mean - ref)
-// in double-float, ref the mean of the partial that holds the maximum; second
-// moments in FP32), so the additions of a pass are independent and nothing
-// waits on a chain of pairwise merges, each with two exponentials and a
-// division.  (With sum w (mean - ref) in FP32 the mean of 2^22 unit normals
-// lost to the pairwise chain: 1.0e-6 against 6.4e-7 of its norm.)
+// Warp `warp` (< kMaxDegrees) merges degree `warp` of G block partials into *out,
+// with its sums S and S2 in double-float (written by several lanes: a barrier
+// before they are read).  Two passes over the partials: the maximum and its
+// index first, then every partial's sums rescaled to that maximum once and
+// added, so the additions of a pass are independent and nothing waits on a
+// chain of pairwise merges, each with two exponentials and a division.  The sums
+// are S, S2, W = sum w (w = S e^(m - M) in FP32: the moments' weight) and, per
+// coefficient, A = sum w d and B = sum (w d^2 + M2), d = mean - ref, ref the mean
+// of the partial that holds the maximum.  The differences d, A, B and B - A^2 / W
+// carry two FP32 words: ref may lie far from the rest of the population (a best
+// trace alone in its block), where B is (distance / deviation)^2 times what is
+// left of it.  In one word that lost 1.6e-3 of the variance at 100 deviations
+// (pairwise merges: 1e-7), and sum w d the mean of 2^22 unit normals by half
+// as much again.
+//
+// This code runs once per launch, by one block, after the kernel's data have
+// streamed through L2: its instructions are fetched cold, so their number is
+// what bounds it.  The loops stay rolled, two coefficients go through one f32x2
+// instruction, and the eight pairs of sums leave the lanes by recursive halving
+// (a lane sends half of what it holds and adds the other half).  The next
+// partial is loaded while the current one is merged; up to 32 are read once,
+// their reference coming from the lane that holds it.  10^5 traces x 32 points,
+// whole call: 34.8 us with B in one word, 34.9 so (36.1 without the pairs); the
+// 4096 uneven sets 10.6 and 9.6 ms (fewer live registers beside their hot loop).
+struct PairSum {  // two sums, each in two words
+  unsigned long long hi, lo;
+};
+
+// a + b; words normalised when a's and b's are
+__device__ __forceinline__ PairSum pair_add(const PairSum& a, const PairSum& b) {
+  const unsigned long long s = f2_add(a.hi, b.hi), bb = f2_sub(s, a.hi);
+  const unsigned long long e = f2_add(f2_sub(a.hi, f2_sub(s, bb)), f2_sub(b.hi, bb));
+  const unsigned long long t = f2_add(e, f2_add(a.lo, b.lo));
+  PairSum r;
+  r.hi = f2_add(s, t);
+  r.lo = f2_sub(t, f2_sub(r.hi, s));
+  return r;
+}
+__device__ __forceinline__ PairSum pair_shfl_xor(const PairSum& a, int o) {
+  return PairSum{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+template <int H>
+__device__ __forceinline__ void halve_sums(PairSum (&v)[8], int lane, int o) {
+  const bool up = lane & o;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const PairSum give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+    v[i] = pair_add(keep, pair_shfl_xor(give, o));
+  }
+}
+
 __device__ __forceinline__ void merge_degree(const DegPartial* parts, int G, int warp, int lane,
-                                             DegPartial& a, DegSums& ds) {
-  // This code runs once per launch, by one block, after the kernel's data
-  // have streamed through L2: its instructions are fetched cold, so the loops
-  // stay rolled (fewer instruction fetches), and the next partial is loaded
-  // while the current one is merged.
-  deg_empty(a);
-  ds.zero();
+                                             DegPartial* out, float2* S_out, float2* S2_out) {
+  constexpr int kP = kMaxCoef / 2;
+  static_assert(kMaxCoef == 6, "the sums make eight pairs");
   const DegPartial* mine = parts + warp;
-  float M = -INFINITY;
-  int arg = 0x7fffffff, at = 0;
+  DegPartial nxt;
+  deg_empty(nxt);
+  if (lane < G) nxt = ld_partial_cg(mine + lane * kMaxDegrees);
+  float M = nxt.m;
+  int arg = nxt.arg, at = lane;
 #pragma unroll 4
-  for (int b = lane; b < G; b += 32) {
+  for (int b = lane + 32; b < G; b += 32) {
     const float2 h = __ldcg(reinterpret_cast<const float2*>(mine + b * kMaxDegrees));
     const int ha = __float_as_int(h.y);
     if (h.x > M || (h.x == M && ha < arg)) {
@@ -269,57 +311,108 @@ __device__ __forceinline__ void merge_degree(const DegPartial* parts, int G, int
       at = ob;
     }
   }
-  if (M == -INFINITY) return;  // the same for the whole warp
-  const DegPartial ref = ld_partial_cg(mine + at * kMaxDegrees);
-  float2 A[kMaxCoef];
-  float B[kMaxCoef];
-#pragma unroll
-  for (int k = 0; k < kMaxCoef; ++k) {
-    A[k] = make_float2(0.0f, 0.0f);
-    B[k] = 0.0f;
+  if (M == -INFINITY) {  // the same for the whole warp
+    if (lane == 0) {
+      deg_empty(*out);
+      *S_out = *S2_out = make_float2(0.0f, 0.0f);
+    }
+    return;
   }
-  DegPartial nxt;
-  if (lane < G) nxt = ld_partial_cg(mine + lane * kMaxDegrees);
+  DegPartial far = nxt;
+  if (G > 32) far = ld_partial_cg(mine + at * kMaxDegrees);
+  const int from = G > 32 ? lane : at;
+  unsigned long long ref[kP];
+#pragma unroll
+  for (int k = 0; k < kP; ++k)
+    ref[k] = __shfl_sync(0xffffffffu, f2_pack(far.mean[2 * k], far.mean[2 * k + 1]), from);
+  PairSum v[8];  // (S, S2), (W, 0), A, B
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i].hi = v[i].lo = 0ull;
 #pragma unroll 1
   for (int b = lane; b < G; b += 32) {
     const DegPartial cur = nxt;
     if (b + 32 < G) nxt = ld_partial_cg(mine + (b + 32) * kMaxDegrees);
     if (cur.m == -INFINITY) continue;
-    const float e = expf(cur.m - M), w = cur.S * e;
-    ds.S = df_add(ds.S, df_prod(cur.S, e));
-    ds.S2 = df_add(ds.S2, df_mul(df_prod(cur.S2, e), e));
+    const float e = expf(cur.m - M);
+    // add x = (hi, lo) to a running sum: the high words' sum exactly, what it
+    // rounds off and the low word in one word
+    auto acc = [](PairSum& a, unsigned long long hi, unsigned long long lo) {
+      const unsigned long long s = f2_add(a.hi, hi), bb = f2_sub(s, a.hi);
+      const unsigned long long r = f2_add(f2_sub(a.hi, f2_sub(s, bb)), f2_sub(hi, bb));
+      a.hi = s;
+      a.lo = f2_add(a.lo, f2_add(r, lo));
+    };
+    const float2 w = df_prod(cur.S, e), s2 = df_mul(df_prod(cur.S2, e), e);
+    acc(v[0], f2_pack(w.x, s2.x), f2_pack(w.y, s2.y));
+    acc(v[1], f2_pack(w.x, 0.0f), 0ull);
+    const unsigned long long ww = f2_pack(w.x, w.x), nw = f2_pack(-w.x, -w.x), ee = f2_pack(e, e);
 #pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) {
-      const float d = cur.mean[k] - ref.mean[k];
-      A[k] = df_add(A[k], df_prod(w, d));
-      B[k] = fmaf(cur.M2[k], e, fmaf(w * d, d, B[k]));
+    for (int k = 0; k < kP; ++k) {
+      // d = mean - ref, t = w d, q = t d in two words (the negated products
+      // give the FMAs their remainders)
+      const unsigned long long mk = f2_pack(cur.mean[2 * k], cur.mean[2 * k + 1]);
+      const unsigned long long d = f2_sub(mk, ref[k]), bb = f2_sub(d, mk);
+      const unsigned long long dl = f2_sub(f2_sub(mk, f2_sub(d, bb)), f2_add(ref[k], bb));
+      const unsigned long long t = f2_mul_rn(ww, d), nt = f2_mul(nw, d);
+      const unsigned long long tl = f2_fma(ww, dl, f2_fma(ww, d, nt));
+      acc(v[2 + k], t, tl);
+      const unsigned long long q = f2_mul_rn(t, d), nq = f2_mul(nt, d);
+      unsigned long long ql = f2_fma(t, dl, f2_fma(tl, d, f2_fma(t, d, nq)));
+      // (second moments are not negative: nothing cancels in their sum)
+      ql = f2_fma(f2_pack(cur.M2[2 * k], cur.M2[2 * k + 1]), ee, ql);
+      acc(v[2 + kP + k], q, ql);
     }
   }
+  halve_sums<4>(v, lane, 16);
+  halve_sums<2>(v, lane, 8);
+  halve_sums<1>(v, lane, 4);
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) v[0] = pair_add(v[0], pair_shfl_xor(v[0], o));
+  // lanes 4 i .. 4 i + 3 hold pair i; lane k < 6 forms coefficient k
+  const float2 th = f2_unpack(v[0].hi), tl = f2_unpack(v[0].lo);
+  const float2 t0 = make_float2(th.x, tl.x), t1 = make_float2(th.y, tl.y);
+  const int k = lane < kMaxCoef ? lane : 0;
+  const float2 S = df_shfl(t0, 0), S2 = df_shfl(t1, 0), W = df_shfl(t0, 4);
+  const int at_a = 8 + 4 * (k / 2), at_b = at_a + 4 * kP;
+  float2 A = df_shfl(t0, at_a), B = df_shfl(t0, at_b);
+  const float2 A1 = df_shfl(t1, at_a), B1 = df_shfl(t1, at_b);
+  if (k & 1) {
+    A = A1;
+    B = B1;
+  }
+  if (lane < kMaxCoef) {
+    float mean = 0.0f, M2 = 0.0f;
+    if (S.x > 0.0f) {
+      const float rk = __ldcg((mine + at * kMaxDegrees)->mean + k);
+      // A / W as the quotient and its remainder; the sum with ref may cancel
+      const float inv = __frcp_rn(W.x), q = __fmul_rn(A.x, inv);
+      const float r = __fadd_rn(__fmaf_rn(-q, W.x, A.x), __fmaf_rn(-q, W.y, A.y));
+      const float2 sh = df_sum(q, __fmul_rn(r, inv));
+      mean = df_add(make_float2(rk, 0.0f), sh).x;
+      M2 = df_add(B, df_neg(df_mul(A, sh))).x;
+      if (M2 < 0.0f) M2 = 0.0f;
+      if (M2 != M2) {
+        // a moment that is not finite, which the low words turn into NaN: its
+        // sum in one word, infinite or NaN as its terms are
+        M2 = 0.0f;
 #pragma unroll 1
-  for (int o = 16; o > 0; o >>= 1) {
-    ds.S = df_add(ds.S, df_shfl_xor(ds.S, o));
-    ds.S2 = df_add(ds.S2, df_shfl_xor(ds.S2, o));
-#pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) {
-      A[k] = df_add(A[k], df_shfl_xor(A[k], o));
-      B[k] += __shfl_xor_sync(0xffffffffu, B[k], o);
+        for (int b = 0; b < G; ++b) {
+          const DegPartial* cur = mine + b * kMaxDegrees;
+          const float e = expf(__ldcg(&cur->m) - M), d = __ldcg(cur->mean + k) - rk;
+          if (e > 0.0f) M2 += fmaf(__ldcg(&cur->S) * e * d, d, __ldcg(cur->M2 + k) * e);
+        }
+      }
     }
+    out->mean[k] = mean;
+    out->M2[k] = M2;
   }
-  a.m = M;
-  a.arg = arg;
-  a.S = ds.S.x;
-  a.S2 = ds.S2.x;
-  if (a.S > 0.0f) {
-    const float inv = __frcp_rn(a.S);
-#pragma unroll
-    for (int k = 0; k < kMaxCoef; ++k) {
-      // ref + A / S with the quotient's and the sum's remainders (they may cancel)
-      const float q = __fmul_rn(A[k].x, inv);
-      const float r = __fadd_rn(__fmaf_rn(-q, ds.S.x, A[k].x), __fmaf_rn(-q, ds.S.y, A[k].y));
-      const float2 mean = df_add(make_float2(ref.mean[k], 0.0f), make_float2(q, __fmul_rn(r, inv)));
-      a.mean[k] = mean.x;
-      a.M2[k] = fmaxf(fmaf(-q, A[k].x, B[k]), 0.0f);
-    }
+  if (lane == 0) {
+    out->m = M;
+    out->arg = arg;
+    out->S = S.x;
+    out->S2 = S2.x;
+    *S_out = S;
+    *S2_out = S2;
   }
 }
 
@@ -329,16 +422,8 @@ __device__ __forceinline__ void finalize_partials(const DegPartial* parts, int G
   __shared__ DegPartial fin[kMaxDegrees];
   __shared__ float2 fS[kMaxDegrees], fS2[kMaxDegrees];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (warp < kMaxDegrees) {
-    DegPartial a;
-    DegSums ds;
-    merge_degree(parts, G, warp, lane, a, ds);
-    if (lane == 0) {
-      fin[warp] = a;
-      fS[warp] = ds.S;
-      fS2[warp] = ds.S2;
-    }
-  }
+  if (warp < kMaxDegrees)
+    merge_degree(parts, G, warp, lane, fin + warp, fS + warp, fS2 + warp);
   __syncthreads();
   if (warp == 0) {
     int32_t st = 0;
@@ -376,16 +461,8 @@ __device__ __forceinline__ void finalize_to_partial(const DegPartial* parts, int
                                                     int min_deg, int64_t N, WsHeader* hdr,
                                                     IsPartial* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (warp < kMaxDegrees) {
-    DegPartial a;
-    DegSums ds;
-    merge_degree(parts, G, warp, lane, a, ds);
-    if (lane == 0) {
-      out->deg[warp] = a;
-      out->S[warp] = ds.S;
-      out->S2[warp] = ds.S2;
-    }
-  }
+  if (warp < kMaxDegrees)
+    merge_degree(parts, G, warp, lane, out->deg + warp, out->S + warp, out->S2 + warp);
   if (threadIdx.x == 0) {
     out->n = N;
     out->n_deg = n_deg;

@@ -80,42 +80,6 @@ __host__ __device__ constexpr size_t trace_smem_bytes() {
   return (sizeof(TraceSmem<PPT>) + 15) / 16 * 16;
 }
 
-// Paired FP32 arithmetic (PTX f32x2, sm_100 and later): two lanes of IEEE
-// single precision in one 64-bit register, each half rounded exactly as the
-// scalar instruction would round it.  One instruction does the work of two,
-// which halves the issue slots of the Horner chain below.
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
-  unsigned long long v;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
-  return v;
-}
-__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
-  float lo, hi;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-  return make_float2(lo, hi);
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // One 32-byte record in a single 256-bit store (sm_100 and later; p 32-byte
 // aligned): a warp's 32 consecutive records are then 32 whole sectors per
 // instruction instead of two half-filled ones each.

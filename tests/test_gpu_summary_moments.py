@@ -1,0 +1,57 @@
+"""Second moments of the posterior summary where the FP32 sums behind them are
+hardest to combine, against FP64."""
+import numpy as np
+import pytest
+
+from gpu_util import load_ppl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ppl():
+    return load_ppl()
+
+
+def _records(n, c):
+    rec = np.zeros((len(n), 8), dtype=np.float32)
+    rec[:, :6] = c
+    rec[:, 6] = n.astype(np.int32).view(np.float32)
+    return rec
+
+
+def _reduce(ppl, n, c, lw):
+    import torch
+    return ppl.read_result(ppl.ppl_posterior_reduce(
+        ppl.poly_model(), torch.from_numpy(_records(n, c)).cuda(), torch.from_numpy(lw).cuda()))
+
+
+# The tiles of 128 particles go round the blocks (one per SM): block 0 holds
+# nothing but each degree's best trace, `dist` standard deviations from the
+# others, which sets the point the final merge works around.  What a block
+# passes on is FP32 (about 1e-6 of its own variance); the merge must not add to
+# it, whatever the distance.
+@pytest.mark.parametrize("dist", [0.0, 10.0, 100.0, 1000.0])
+def test_best_trace_alone_in_its_block(ppl, orc, dist):
+    import torch
+    blocks = torch.cuda.get_device_properties(0).multi_processor_count
+    N = blocks * 128 * 64
+    rng = np.random.default_rng(17)
+    n = rng.integers(2, 6, N)
+    c = rng.standard_normal((N, 6)).astype(np.float32)
+    lw = rng.uniform(-1.5, -0.5, N).astype(np.float32)
+    lw[(np.arange(N) // 128) % blocks == 0] = -np.inf
+    for d in range(4):
+        i = 7 + 30 * d
+        n[i], lw[i], c[i] = 2 + d, 0.0, dist
+    c[np.arange(6)[None, :] > n[:, None]] = 0
+    out = _reduce(ppl, n, c, lw)
+    ref = orc.posterior_poly(orc.poly_model(), lw.astype(np.float64), n.astype(np.int32),
+                             c.astype(np.float64))
+    assert out["status"] == 0 and list(out["deg_argmax"]) == [7, 37, 67, 97]
+    for d in range(4):
+        live = slice(0, d + 3)
+        var = ref["deg_var"][d][live]
+        assert np.all(np.abs(out["deg_var"][d][live] - var) <= 1e-5 * var), (d, out["deg_var"][d], var)
+        err = np.abs(out["deg_mean"][d][live] - ref["deg_mean"][d][live])
+        assert np.all(err <= 1e-6 * (np.sqrt(var) + np.abs(ref["deg_mean"][d][live])))
