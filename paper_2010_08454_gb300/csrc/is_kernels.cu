@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kPostThreads, 1) posterior_kernel(
 #pragma unroll 1
     for (int o = 1; o < kPostWarps; o <<= 1) {
       const DegPartial other = deg_shfl_xor(r, o);
-      deg_merge(r, other);
+      deg_merge<true>(r, other);
     }
     if (lane == 0) parts[blockIdx.x * kMaxDegrees + warp] = r;
   }

@@ -2,8 +2,14 @@
 // in registers as f32x2 pairs around a reference that the lanes of a warp
 // share: S = sum w, S2 = sum w^2, A = sum w d, B = sum w d^2, with w = exp(lw -
 // m_ref) and d = c - ref.  A trace is added to all four degrees with its
-// weight masked (28 paired multiply-adds: no shuffle and no branch on the
+// weight masked (40 paired operations: no shuffle and no branch on the
 // degree); when the reference moves, the sums move with it exactly.
+//
+// Squares are formed as (w d) d and never as w (d d): d^2 leaves FP32's range at
+// |d| = 1.8e19, and its product with another degree's zero weight would be a NaN
+// in that degree's sums.  (With d^2 shared by the degrees 31 operations: 2^24
+// records summarised and resampled 435 us against 438 so, 1024 sets x 2^16 traces
+// under their proposals 1987 against 2003.)
 #pragma once
 
 #include "posterior.cuh"
@@ -35,9 +41,6 @@ __device__ __forceinline__ void lane_add(LaneSums (&a)[kMaxDegrees], int d, floa
       f2_sub(f2_pack(c[0], c[1]), f2_pack(f0.x, f0.y)),
       f2_sub(f2_pack(c[2], c[3]), f2_pack(f0.z, f0.w)),
       f2_sub(f2_pack(c[4], c[5]), f2_pack(f1.x, f1.y))};
-  unsigned long long q2[kMaxCoef / 2];
-#pragma unroll
-  for (int j = 0; j < kMaxCoef / 2; ++j) q2[j] = f2_mul(d2[j], d2[j]);
   const unsigned long long one_w = f2_pack(1.0f, w);
 #pragma unroll
   for (int k = 0; k < kMaxDegrees; ++k) {
@@ -47,24 +50,26 @@ __device__ __forceinline__ void lane_add(LaneSums (&a)[kMaxDegrees], int d, floa
 #pragma unroll
     for (int j = 0; j < kMaxCoef / 2; ++j) {
       a[k].A[j] = f2_fma(ww, d2[j], a[k].A[j]);
-      a[k].B[j] = f2_fma(ww, q2[j], a[k].B[j]);
+      a[k].B[j] = f2_fma(f2_mul(ww, d2[j]), d2[j], a[k].B[j]);
     }
   }
 }
 
 // Move a lane's sums to a reference g below the old one (g = old - new per
-// coefficient), rescaling the weights by ex.
+// coefficient), rescaling the weights by ex (first: a reference far away that
+// carried a negligible weight moves without leaving FP32's range).
 __device__ __forceinline__ void lane_move(LaneSums& a, const float (&g)[kMaxCoef], float ex) {
   const float2 s = f2_unpack(a.s12);
-  const unsigned long long ee = f2_pack(ex, ex), ss = f2_pack(s.x, s.x);
+  const float es = s.x * ex;
+  const unsigned long long ee = f2_pack(ex, ex), ss = f2_pack(es, es);
 #pragma unroll
   for (int j = 0; j < kMaxCoef / 2; ++j) {
-    const unsigned long long gg = f2_pack(g[2 * j], g[2 * j + 1]);
-    const unsigned long long A1 = f2_fma(ss, gg, a.A[j]);  // A + S g
-    a.B[j] = f2_mul(ee, f2_fma(gg, f2_add(a.A[j], A1), a.B[j]));
-    a.A[j] = f2_mul(ee, A1);
+    const unsigned long long gg = f2_pack(g[2 * j], g[2 * j + 1]), A0 = f2_mul(ee, a.A[j]);
+    const unsigned long long A1 = f2_fma(ss, gg, A0);  // A + S g
+    a.B[j] = f2_fma(gg, f2_add(A0, A1), f2_mul(ee, a.B[j]));
+    a.A[j] = A1;
   }
-  a.s12 = f2_pack(s.x * ex, s.y * ex * ex);
+  a.s12 = f2_pack(es, s.y * ex * ex);
 }
 
 // The warp's partial of one degree in every lane: its lanes' sums around ref

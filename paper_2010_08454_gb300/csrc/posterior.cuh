@@ -38,7 +38,12 @@ __device__ __forceinline__ void deg_empty(DegPartial& p) {
   }
 }
 
-// a <- merge(a, b)
+// a <- merge(a, b).  kFar: for partials of small groups, one of which may hold
+// nothing but a trace far away with next to no weight: the mean moves from the
+// heavier side's, and squares are weighted before they are formed (d^2 leaves
+// FP32's range at 1.8e19).  The trace kernels' folds, whose coefficients come
+// from the prior, do without (their last bits, and 1 % of their time).
+template <bool kFar = false>
 __device__ __forceinline__ void deg_merge(DegPartial& a, const DegPartial& b) {
   if (b.m == -INFINITY) return;
   if (a.m == -INFINITY) {
@@ -49,11 +54,14 @@ __device__ __forceinline__ void deg_merge(DegPartial& a, const DegPartial& b) {
   const float ea = expf(a.m - M), eb = expf(b.m - M);
   const float wa = a.S * ea, wb = b.S * eb, w = wa + wb;
   const float fb = wb / w, cross = wa * fb;
+  const bool from_b = kFar && wb > wa;
+  const float f = from_b ? -(wa / w) : fb;
 #pragma unroll
   for (int k = 0; k < kMaxCoef; ++k) {
     const float d = b.mean[k] - a.mean[k];
-    a.mean[k] = fmaf(d, fb, a.mean[k]);
-    a.M2[k] = fmaf(d * d, cross, fmaf(a.M2[k], ea, b.M2[k] * eb));
+    a.mean[k] = fmaf(d, f, from_b ? b.mean[k] : a.mean[k]);
+    const float m2 = fmaf(a.M2[k], ea, b.M2[k] * eb);
+    a.M2[k] = kFar ? fmaf(d * cross, d, m2) : fmaf(d * d, cross, m2);
   }
   a.S2 = fmaf(a.S2, ea * ea, b.S2 * eb * eb);
   a.S = w;

@@ -55,3 +55,32 @@ def test_best_trace_alone_in_its_block(ppl, orc, dist):
         assert np.all(np.abs(out["deg_var"][d][live] - var) <= 1e-5 * var), (d, out["deg_var"][d], var)
         err = np.abs(out["deg_mean"][d][live] - ref["deg_mean"][d][live])
         assert np.all(err <= 1e-6 * (np.sqrt(var) + np.abs(ref["deg_mean"][d][live])))
+
+
+# One coefficient whose square leaves FP32's range: with a weight that FP32
+# rounds to 0, or one that makes it the whole variance of its own degree; in the
+# midst of others, and as the first of its degree that its warp meets (where it
+# sets the point that the warp's sums are taken around).
+@pytest.mark.parametrize("first", [False, True])
+@pytest.mark.parametrize("lw_far", [-300.0, -69.0])
+def test_coefficient_whose_square_overflows(ppl, orc, lw_far, first):
+    N, at = 40000, 5
+    rng = np.random.default_rng(3)
+    n = rng.integers(2, 6, N)
+    c = rng.standard_normal((N, 6)).astype(np.float32)
+    lw = rng.uniform(-1.5, 0.0, N).astype(np.float32)
+    n[:128] = 3
+    if first:
+        n[:128] = np.where(np.arange(128) % 2 == 0, 2, 4)
+    n[at] = 3
+    c[np.arange(6)[None, :] > n[:, None]] = 0
+    c[at, 1] = 1e20
+    lw[at] = lw_far
+    out = _reduce(ppl, n, c, lw)
+    ref = orc.posterior_poly(orc.poly_model(), lw.astype(np.float64), n.astype(np.int32),
+                             c.astype(np.float64))
+    assert out["status"] == 0
+    for d in range(4):
+        live = slice(0, d + 3)
+        var = ref["deg_var"][d][live]
+        assert np.all(np.abs(out["deg_var"][d][live] - var) <= 1e-5 * var), (d, out["deg_var"][d], var)
