@@ -84,3 +84,20 @@ def test_coefficient_whose_square_overflows(ppl, orc, lw_far, first):
         live = slice(0, d + 3)
         var = ref["deg_var"][d][live]
         assert np.all(np.abs(out["deg_var"][d][live] - var) <= 1e-5 * var), (d, out["deg_var"][d], var)
+
+
+# A moment that FP32 cannot hold is reported as such: a NaN coefficient that
+# carries weight shows in its variance as in its mean, and one of 1e20
+# with an ordinary weight gives no finite variance.
+@pytest.mark.parametrize("N", [100, 5000])
+@pytest.mark.parametrize("value", [float("nan"), 1e20])
+def test_moments_out_of_range_are_not_hidden(ppl, value, N):
+    rng = np.random.default_rng(4)
+    n = np.full(N, 3)
+    c = rng.standard_normal((N, 6)).astype(np.float32)
+    c[:, 4:] = 0
+    c[N // 2, 1] = value
+    out = _reduce(ppl, n, c, np.zeros(N, dtype=np.float32))
+    assert not np.isfinite(out["deg_var"][1][1])
+    assert np.isnan(out["deg_mean"][1][1]) == np.isnan(value)
+    assert np.all(np.isfinite(out["deg_var"][1][[0, 2, 3]]))
