@@ -59,8 +59,13 @@ __device__ __forceinline__ void load_proposal(const PolyParams& p, const float* 
   if (lane < kMaxSlots && lane < base) {
     const float t = fminf(fmaxf(o[5 + 2 * lane], -9.0f), 1.0f);
     const float s = p.prior_sigma * expf(t);
-    // (1 / s is the prior's reciprocal when s equals sigma)
-    ps.slot[lane] = make_float4(p.prior_sigma * o[4 + 2 * lane], s, 1.0f / s, log_sigma + t);
+    const float mu = p.prior_sigma * o[4 + 2 * lane];
+    // (1 / s is the prior's reciprocal when s equals sigma).  Where the mean is NaN
+    // or infinite, the density is NaN and the draws are made around 0: every such
+    // trace has a NaN log-weight as before, but no coefficient that 0 x NaN would
+    // carry into other degrees' sums.
+    const bool ok = fabsf(mu) < INFINITY;
+    ps.slot[lane] = make_float4(ok ? mu : 0.0f, s, 1.0f / s, ok ? log_sigma + t : NAN);
   }
 }
 

@@ -3,6 +3,7 @@ hardest to combine, against FP64."""
 import numpy as np
 import pytest
 
+import synth
 from gpu_util import load_ppl
 
 pytestmark = pytest.mark.gpu
@@ -101,3 +102,34 @@ def test_moments_out_of_range_are_not_hidden(ppl, value, N):
     assert not np.isfinite(out["deg_var"][1][1])
     assert np.isnan(out["deg_mean"][1][1]) == np.isnan(value)
     assert np.all(np.isfinite(out["deg_var"][1][[0, 2, 3]]))
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_nan_traces_of_one_degree_leave_the_others(ppl, value):
+    # a proposal whose third degree holds a NaN mean (or an infinite one), in a batch large enough for the
+    # kernel that keeps lane sums: the status tells, and the other degrees'
+    # moments are those of the same proposal without it, bit for bit
+    import torch
+    sets, N = 4, 1 << 23
+    d = synth.prior_datasets(sets, 16, 5)
+    doff, poff = np.arange(sets + 1) * 16, np.arange(sets + 1) * N
+    model = ppl.poly_model()
+    ws = ppl.batched_workspace(doff, poff)
+    plan = ppl.ppl_batched_prepare(model, doff, poff, 8, 2, ws)
+    x, y = (torch.from_numpy(np.ascontiguousarray(d[k], dtype=np.float32).reshape(-1)).cuda() for k in "xy")
+    do, po = torch.from_numpy(doff).cuda(), torch.from_numpy(poff).cuda()
+    prop = torch.zeros((sets, 48), device="cuda")
+    rows = []
+    for bad in (False, True):
+        if bad:
+            prop[1, 4 + 2 * 7] = value  # degrees 2 and 3 take 3 + 4 slots
+        out = ppl.batch_results_tensor(sets)
+        ppl.ppl_infer_is_learned(model, x, y, do, po, 7, plan, prop, out, ws)
+        assert ppl.ppl_batched_status(ws) == (ppl.PPL_ENAN if bad else 0)
+        rows.append(ppl.read_batch_results(out, sets))
+    good, bad = rows
+    for f in ("deg_mean", "deg_var", "deg_argmax"):
+        assert np.array_equal(good[0][f], bad[0][f]) and np.array_equal(good[3][f], bad[3][f])
+        others = [0, 1, 3]
+        assert np.array_equal(np.asarray(good[1][f])[others], np.asarray(bad[1][f])[others]), f
+    assert bad[1]["deg_argmax"][2] == -1 and bad[1]["p_n"][2] == 0.0
