@@ -247,7 +247,9 @@ ppl_status ppl_resample_shard_plan(const uint64_t* totals, int32_t n_shards, int
  * k_first].  With state_in [dev, n_local records of stride_bytes, a multiple
  * of 4 up to 1024, 4-byte aligned] the records of those outputs' ancestors
  * are copied to state_out [dev, k_end - k_first records].  `plan` [host] is
- * this shard's entry.  Workspace: ppl_workspace_size(any model, n_local, 0). */
+ * this shard's entry; one that does not belong to these weights (its outputs
+ * are not those that their sums cover) sets PPL_EINVAL in the workspace status,
+ * and nothing is written.  Workspace: ppl_workspace_size(any model, n_local, 0). */
 ppl_status ppl_resample_shard(const float* lw, int64_t n_local, int64_t first_particle,
                               const double* max_lw_dev, const ppl_resample_plan* plan,
                               int32_t* ancestors, const void* state_in, int64_t stride_bytes,

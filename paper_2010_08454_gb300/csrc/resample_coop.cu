@@ -429,10 +429,19 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
     const uint64_t T = warp_sum_acc<false>(lane < kRcWarps ? jtot[lane] : 0ull);
     bool valid;
     uint64_t stride = 0, u = 0;
-    if (a.planned) {  // a shard: the population's layout is given
-      valid = T <= (1ull << 61) && a.p_stride > 0;
+    if (a.planned) {
+      // a shard: the population's layout is given, and has to be the one of these
+      // weights, since the outputs' places and number follow from both: the first
+      // output at or above this shard's prefix and the first past its end
       stride = a.p_stride;
       u = a.p_u;
+      constexpr uint64_t kMost = 1ull << 61;
+      valid = stride > 0 && stride <= kMost && u < stride && T <= kMost && a.c_base <= kMost - T;
+      if (valid) {
+        const DivInv sv = div_inv(stride);
+        valid = positions_below_inv(a.c_base, u, sv, a.m) == a.k_off &&
+                positions_below_inv(a.c_base + T, u, sv, a.m) == a.k_end;
+      }
     } else {
       valid = T > 0 && T <= (1ull << 61) && T >= (uint64_t)a.m;
       if (valid) {
@@ -641,7 +650,10 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         const int32_t mk = marks[j0 + lane];
         marks[j0 + lane] = 0;
         const unsigned at = __ballot_sync(0xffffffffu, mk != 0) & (0xffffffffu >> (31 - lane));
-        const int an = (int)cb + __shfl_sync(0xffffffffu, mk, 31 - __clz(at)) - 1;
+        // (every row's first output is marked: the chunk's outputs are those that its
+        // own sums cover; the bound keeps an access inside the records all the same)
+        const int src = __shfl_sync(0xffffffffu, mk, 31 - __clz(at)) - 1;
+        const int an = (int)cb + min(max(src, 0), nCw - 1);
         if (lane < n) a.anc[k0 + lane] = an + (int32_t)a.j_off;
         if constexpr (REC == kRec32) {
           if (lane < n)

@@ -1,0 +1,59 @@
+"""The resampler's scatter form (row marks) at the edges of its rows, records
+and plans."""
+import numpy as np
+import pytest
+
+import synth
+from gpu_util import load_ppl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ppl():
+    return load_ppl()
+
+
+# A shard's plan says where its outputs lie; one that its weights do not bear out
+# is refused and writes nothing (the buffers hold room for what it claims).
+@pytest.mark.parametrize("change", ["none", "k_end+1", "k_end-1", "k_first+1", "k_first-1", "c_base",
+                                    "stride", "offset", "weights"])
+@pytest.mark.parametrize("N,M", [(40000, 40000), (5000, 1 << 20)])
+def test_plan_that_does_not_fit_the_weights(ppl, N, M, change):
+    import torch
+    lw = torch.from_numpy(synth.log_weights(N, 9, "normal", scale=1.0)).cuda()
+    h = N // 2 + 77
+    mx = lw.max().double().reshape(1)
+    shards = [lw[:h].clone(), lw[h:].clone()]
+    totals = [int(ppl.ppl_resample_shard_total(s, mx, N).item()) for s in shards]
+    plan = ppl.ppl_resample_shard_plan(np.array(totals, dtype=np.uint64), N, M, 3)[1]
+    n_out = plan.k_end - plan.k_first
+    anc = torch.full((n_out + 512,), -7, dtype=torch.int32, device="cuda")
+    rec = torch.arange(8 * (N - h), dtype=torch.float32, device="cuda").view(N - h, 8)
+    out = torch.full((n_out + 512, 8), -7.0, device="cuda")
+    if change == "k_end+1":
+        plan.k_end, plan.m = plan.k_end + 1, plan.m + 1
+    elif change == "k_end-1":
+        plan.k_end -= 1
+    elif change == "k_first+1":
+        plan.k_first += 1
+    elif change == "k_first-1":
+        plan.k_first -= 1
+    elif change == "c_base":
+        plan.c_base += 2 * plan.stride
+    elif change == "stride":
+        plan.stride += plan.stride // 2
+    elif change == "offset":
+        plan.offset = plan.stride
+    elif change == "weights":
+        shards[1][100] -= 5.0
+        shards[1][1000:1100] -= 1.0
+    ws = ppl.workspace(ppl.poly_model(), N)
+    ppl.ppl_resample_shard(shards[1], h, mx, plan, ancestors=anc, state_in=rec, state_out=out, ws=ws)
+    if change == "none":
+        assert ppl.ppl_workspace_status(ws) == 0
+        assert torch.equal(out[:n_out], rec[anc[:n_out].long() - h])
+    else:
+        assert ppl.ppl_workspace_status(ws) == ppl.PPL_EINVAL
+        assert bool((anc == -7).all()) and bool((out == -7.0).all())
+    assert bool((anc[n_out:] == -7).all()) and bool((out[n_out:] == -7.0).all())
