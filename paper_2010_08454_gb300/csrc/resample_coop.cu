@@ -357,6 +357,10 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
   __shared__ int64_t seg_sh[2][6];  // chunk, its first and end unit, first and end output, C at its start
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned G = gridDim.x;
+  // runs that reach more than one later row: each takes over 32 of the chunk's outputs
+  __shared__ int3 long_runs[kRcScatterOut / 32];
+  __shared__ int n_long;
+  if (tid == 0) n_long = 0;
   bool cleared = false;  // the marks, before the block's first scattered chunk
   float m_lw = 0.0f, scale = 0.0f;
   if (FROM_LW) {
@@ -614,7 +618,11 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         // particles and marks, in the chunk's output table, each one's first
         // offspring and the first output of every later row of 32 that its
         // offspring reach: a slot's ancestor is then the last mark at or
-        // before it in its own row.
+        // before it in its own row.  The thread marks the next row alone; the
+        // rest of a long run goes to a warp (marked by the thread while the block
+        // waits, 10^4 particles with log-weights of deviation 10: 39.3 us
+        // against 36.1; near-uniform 10^5 x 24 B 39.1 and 40.0, 2^24 x 32 B 303 and
+        // 305, where the runs end in their row or the next).
         const int n_out = (int)(kn - kc);
         const StepDiv dv(u + (uint64_t)kc * stride, stride);
         int k0 = min(dv.below(base), n_out);
@@ -624,7 +632,12 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
           if (k1 > k0) {
             const int32_t mark = (int32_t)(tid * kRcItems + r) + 1;
             marks[k0] = mark;
-            for (int row = k0 / 32 + 1; row * 32 < k1; ++row) marks[row * 32] = mark;
+            const int e = (k0 | 31) + 1;
+            if (e < k1) {
+              marks[e] = mark;
+              if (e + 32 < k1)  // more rows: left to a warp
+                long_runs[atomicAdd(&n_long, 1)] = make_int3(e + 32, k1, mark);
+            }
           }
           k0 = k1;
         }
@@ -636,6 +649,14 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         if ((tid & 31) == 31) sL1[tid >> 5] = last;  // thread 32 i + 31 ends 256-block i
       }
       __syncthreads();
+      if (n_long > 0) {  // the same for the whole block
+        for (int e = warp; e < n_long; e += kRcWarps) {
+          const int3 w = long_runs[e];
+          for (int q = w.x + 32 * lane; q < w.y; q += 32 * 32) marks[q] = w.z;
+        }
+        __syncthreads();
+        if (tid == 0) n_long = 0;  // (a barrier lies before the next chunk's runs)
+      }
     }
     // warp 0 fetches the next chunk's descriptor while the others take this
     // chunk's items

@@ -57,3 +57,30 @@ def test_plan_that_does_not_fit_the_weights(ppl, N, M, change):
         assert ppl.ppl_workspace_status(ws) == ppl.PPL_EINVAL
         assert bool((anc == -7).all()) and bool((out == -7.0).all())
     assert bool((anc[n_out:] == -7).all()) and bool((out[n_out:] == -7.0).all())
+
+
+def _gather_check(ppl, orc, lw, M, state, seed=13):
+    import torch
+    st, ref = orc.resample_from_lw(lw, M, seed, 1, 3)
+    assert st == 0
+    anc, out = ppl.ppl_resample_gather(M, seed, torch.from_numpy(lw).cuda(), state, instance=1, t=3)
+    assert np.array_equal(anc.cpu().numpy(), ref)
+    assert torch.equal(out.view(torch.uint8), state[anc.long()].view(torch.uint8))
+
+
+# Runs of one particle's offspring over none, one, several and all rows of its
+# chunk, several long runs at once, and up to the most outputs that a chunk
+# writes in this form (8192).
+@pytest.mark.parametrize("M", [33, 4096, 7001, 8192, 8193, 20000])
+@pytest.mark.parametrize("N", [1, 40, 4096, 10000])
+def test_runs_over_many_rows(ppl, orc, N, M):
+    import torch
+    rng = np.random.default_rng([N, M])
+    state = torch.from_numpy(rng.standard_normal((N, 6)).astype(np.float32)).cuda()
+    for scale in (0.5, 4.0, 10.0, 40.0):
+        _gather_check(ppl, orc, (scale * rng.standard_normal(N)).astype(np.float32), M, state)
+    lw = np.full(N, -np.inf, dtype=np.float32)
+    lw[N // 2] = 0.0  # one particle takes everything
+    _gather_check(ppl, orc, lw, M, state)
+    lw[:] = -1.25     # all alike: runs of M / N
+    _gather_check(ppl, orc, lw, M, state)
