@@ -84,3 +84,45 @@ def test_runs_over_many_rows(ppl, orc, N, M):
     _gather_check(ppl, orc, lw, M, state)
     lw[:] = -1.25     # all alike: runs of M / N
     _gather_check(ppl, orc, lw, M, state)
+
+
+# Records of every kind the fused gather distinguishes: 4-byte words past one
+# round of a row's copies, the widest record, 32-byte records that lie 4 or 16
+# bytes off a 32-byte boundary; near-uniform and concentrated weights, rows and
+# chunks that end ragged.
+@pytest.mark.parametrize("words,shift", [(5, 0), (6, 0), (7, 0), (255, 0), (256, 0), (8, 1), (8, 4),
+                                         (12, 0), (12, 2), (4, 4)])
+@pytest.mark.parametrize("N,M", [(4099, 4099), (9000, 17999), (5000, 4097)])
+def test_record_kinds(ppl, orc, words, shift, N, M):
+    import torch
+    rng = np.random.default_rng([N, words])
+    def room(n):
+        return torch.empty(n * words + shift, device="cuda")[shift:].view(n, words)
+    state, out = room(N), room(M)
+    state.copy_(torch.from_numpy(rng.standard_normal((N, words)).astype(np.float32)))
+    for lw in (np.full(N, -1.25, dtype=np.float32), synth.log_weights(N, 5, "normal", scale=0.3),
+               synth.log_weights(N, 6, "normal", scale=12.0)):
+        st, ref = orc.resample_from_lw(lw, M, 13, 1, 3)
+        assert st == 0
+        anc, got = ppl.ppl_resample_gather(M, 13, torch.from_numpy(lw).cuda(), state, state_out=out,
+                                           instance=1, t=3)
+        assert np.array_equal(anc.cpu().numpy(), ref)
+        assert got.data_ptr() == out.data_ptr() and torch.equal(out, state[anc.long()])
+
+
+@pytest.mark.parametrize("words", [6, 12])
+def test_sharded_gather_of_other_records(ppl, words):
+    import torch
+    N, M = 30011, 30011
+    lw = torch.from_numpy(synth.log_weights(N, 9, "normal", scale=1.0)).cuda()
+    state = torch.randn(N, words, device="cuda")
+    anc_ref, rec_ref = ppl.ppl_resample_gather(M, 3, lw, state)
+    b = [0, 11000, 11001, N]
+    mx = lw.max().double().reshape(1)
+    parts = [lw[b[g]:b[g + 1]].clone() for g in range(3)]
+    totals = [int(ppl.ppl_resample_shard_total(p, mx, N).item()) for p in parts]
+    plans = ppl.ppl_resample_shard_plan(np.array(totals, dtype=np.uint64), N, M, 3)
+    got = [ppl.ppl_resample_shard(parts[g], b[g], mx, plans[g],
+                                  state_in=state[b[g]:b[g + 1]].clone()) for g in range(3)]
+    assert torch.equal(torch.cat([g[0] for g in got]), anc_ref)
+    assert torch.equal(torch.cat([g[1] for g in got]), rec_ref)
