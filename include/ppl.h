@@ -439,14 +439,17 @@ ppl_status ppl_rng_words(uint64_t seed, uint32_t instance, uint32_t step, uint32
  * its draws use counter field instance = b.  The work is cut into (instance,
  * tile of 256 * ppt particles) items taken heaviest first (longest data first)
  * from an atomic queue by num_SMs * blocks_per_sm resident blocks; the last
- * item of an instance writes out_dev[b] [dev].
+ * item of an instance writes out_dev[b] [dev].  Large batches of short data sets
+ * (at most 32 points each, 2^25 particles in all, 16384 a set on average) go
+ * through the tiles in instance order instead, with two blocks per SM.
  *  ppl_batched_workspace_size: bytes for any configuration (host offsets).
  *  ppl_batched_prepare: builds the item plan on the host from host copies of
  *    the offsets, copies it into `ws` and synchronises `stream`; fills *plan.
  *  ppl_infer_is_batched: the launch (a memset, a device copy and one kernel);
  *    it can be captured in a CUDA graph and replayed.
  *  ppl_batched_autotune: times every ppt in {1,2,4,8} x blocks_per_sm in
- *    {1..4} on the caller's data, keeps the fastest (cached as one JSON line in
+ *    {1..4} (2 alone for the large batches above) on the caller's data, keeps the
+ *    fastest (cached as one JSON line in
  *    cache_path, reused when the batch's shape matches), and prepares it. */
 typedef struct {
   int32_t ppt, blocks_per_sm, n_inst, pad;

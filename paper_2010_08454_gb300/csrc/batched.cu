@@ -397,12 +397,18 @@ __global__ void __launch_bounds__(kTpb, 2) lanes_kernel(
   }
 }
 
+// Whether a batch runs in lanes_kernel (which takes two blocks per SM, whatever
+// the plan says).
+static bool in_lanes(int64_t max_len, int64_t total, int32_t n_inst) {
+  return max_len <= kLanesMaxLen && total >= kLanesMinTotal && total / n_inst >= kLanesMinMean;
+}
+
 template <int PPT, bool LEARNED>
 static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const float* y,
                                     const int64_t* data_off, const int64_t* part_off,
-                                    int32_t n_inst, int64_t n_items, int64_t max_len, int64_t total, int blocks_per_sm,
-                                    uint64_t seed, const float* proposal, char* ws,
-                                    ppl_is_result* out, cudaStream_t s) {
+                                    int32_t n_inst, int64_t n_items, int64_t max_len, int64_t total,
+                                    int blocks_per_sm, uint64_t seed, const float* proposal,
+                                    char* ws, ppl_is_result* out, cudaStream_t s) {
   const BatchLayout l = batch_layout(n_items, n_inst);
   WsHeader* hdr = reinterpret_cast<WsHeader*>(ws + l.header);
   cudaError_t e = cudaMemsetAsync(ws + l.header, 0, 512, s);
@@ -412,7 +418,7 @@ static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const f
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(ws + l.inst_max, 0, (size_t)n_inst * kMaxDegrees * sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
-  if (max_len <= kLanesMaxLen && total >= kLanesMinTotal && total / n_inst >= kLanesMinMean) {
+  if (in_lanes(max_len, total, n_inst)) {
     const int64_t blocks = (int64_t)num_sms() * 2;
     const int run = (int)std::max<int64_t>(1, kRunTraces / (kTpb * PPT));
     const int64_t runs = (n_items + run - 1) / run;
@@ -445,16 +451,17 @@ static cudaError_t launch_batched_t(const PolyParams& p, const float* x, const f
 
 cudaError_t launch_batched(const PolyParams& p, const float* x, const float* y,
                            const int64_t* data_off, const int64_t* part_off, int32_t n_inst,
-                           int64_t n_items, int64_t max_len, int64_t total, int ppt, int blocks_per_sm, uint64_t seed,
-                           const float* proposal, char* ws, ppl_is_result* out, cudaStream_t s) {
+                           int64_t n_items, int64_t max_len, int64_t total, int ppt,
+                           int blocks_per_sm, uint64_t seed, const float* proposal, char* ws,
+                           ppl_is_result* out, cudaStream_t s) {
 #define PPL_BATCHED_CASE(P)                                                                   \
   case P:                                                                                     \
-    return proposal ? launch_batched_t<P, true>(p, x, y, data_off, part_off, n_inst, n_items, max_len, total, \
-                                                blocks_per_sm, seed, proposal, ws, out, s)    \
-                    : launch_batched_t<P, false>(p, x, y, data_off, part_off, n_inst,         \
-                                                 n_items, max_len, total, blocks_per_sm, seed, \
-                                                 nullptr, ws,                                 \
-                                                 out, s);
+    return proposal ? launch_batched_t<P, true>(p, x, y, data_off, part_off, n_inst, n_items, \
+                                                max_len, total, blocks_per_sm, seed, proposal, \
+                                                ws, out, s)                                   \
+                    : launch_batched_t<P, false>(p, x, y, data_off, part_off, n_inst, n_items, \
+                                                 max_len, total, blocks_per_sm, seed, nullptr, \
+                                                 ws, out, s);
   switch (ppt) {
     PPL_BATCHED_CASE(1)
     PPL_BATCHED_CASE(2)
@@ -640,6 +647,7 @@ ppl_status ppl_batched_status(const void* ws, ppl_stream stream) {
 }
 
 // Autotuner: times every (ppt, blocks_per_sm) candidate on the caller's data
+// (every ppt where the kernel has its own number of blocks)
 // (two warm-up launches, then the median of three), keeps the fastest, and
 // records it in `cache_path` (a one-line JSON object keyed by the batch's
 // shape).  A cached entry with the same key is reused without timing.
@@ -687,8 +695,10 @@ ppl_status ppl_batched_autotune(const ppl_model* model, const float* x, const fl
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return PPL_ECUDA;
+  const bool lanes = in_lanes(max_len, part_off_host[n_inst], n_inst);
   for (int ppt : ppts) {
     for (int bps : bpss) {
+      if (lanes && bps != 2) continue;  // the same launch
       ppl_batch_plan plan;
       ppl_status st = ppl_batched_prepare(model, data_off_host, part_off_host, n_inst, ppt, bps,
                                           &plan, ws, ws_bytes, stream);

@@ -68,3 +68,21 @@ def test_learned_proposals_across_runs(ppl, orc, ppt):
     for b in range(n, n + len(big)):
         assert large[b]["status"] == 0 and large[b]["n_particles"] == big[b - n]
         assert np.isfinite(large[b]["log_z"]) and large[b]["ess"] > 0
+
+
+def test_autotuner_times_one_number_of_blocks(ppl, tmp_path):
+    # the kernel of large batches has its own number of blocks: the candidates that
+    # differ in nothing else are one launch, timed once
+    import torch
+    B, N = 64, 1 << 19
+    d = synth.prior_datasets(B, 16, 3)
+    doff, poff = np.arange(B + 1) * 16, np.arange(B + 1) * N
+    t = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in
+         (d["x"].astype(np.float32).reshape(-1), d["y"].astype(np.float32).reshape(-1), doff, poff)]
+    model = ppl.poly_model()
+    ws = ppl.batched_workspace(doff, poff)
+    out = ppl.batch_results_tensor(B)
+    for k in range(4):
+        plan = ppl.ppl_batched_autotune(model, *t, doff, poff, k, out, ws,
+                                        str(tmp_path / f"tune{k}.json"))
+        assert plan.blocks_per_sm == 2
