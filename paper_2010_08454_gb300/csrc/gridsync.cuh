@@ -166,9 +166,14 @@ __device__ __forceinline__ int64_t positions_below_inv(uint64_t c, uint64_t u, c
 }
 
 // Division of the resampling positions by their stride when the quotient is
-// small: k(c) = #{j >= 0 : pos0 + j stride < c} for c - pos0 <= 2^16 stride
-// (more outputs than a block's table or a cluster holds); beyond, some count
-// that is at least as large as 2^15.
+// small: k(c) = #{j >= 0 : pos0 + j stride < c}, exact up to 2^16 (more outputs
+// than a block's table or a cluster holds), and some count of at least 2^15
+// beyond, for (c - pos0) >> sh < 2^32 (sh: the stride's bits past 16).  Callers
+// count from an output k of their own and pass prefix sums that end at most
+// 2^15 outputs on, or, past the last of m outputs, at most the division's
+// remainder T - m stride < m < 2^31 further: 2^15 strides < 2^31 << sh, and the
+// remainder < 2^31.  The count may pass 2^31 there (stride 1), so it is unsigned,
+// and callers bound it before they index with it.
 // With the stride's leading 16 bits the quotient's FP32 estimate is within
 // one of the exact one, and one remainder settles it: 15 instructions where
 // the general division of two 64-bit integers takes about 50.
@@ -180,13 +185,13 @@ struct StepDiv {
     sh = max(0, 48 - __clzll(s));  // s >> sh < 2^16
     inv = __frcp_rn(lead_f32(s) * __int_as_float((127 - sh) << 23));
   }
-  __device__ __forceinline__ int below(uint64_t c) const {
+  __device__ __forceinline__ uint32_t below(uint64_t c) const {
     if (c <= pos0) return 0;
     const uint64_t num = c - pos0 - 1;
     int64_t q = (int64_t)__float2uint_rz(__uint2float_rz((uint32_t)(num >> sh)) * inv);
     const int64_t r = (int64_t)(num - (uint64_t)q * stride);
     q += r < 0 ? -1 : (r >= (int64_t)stride ? 1 : 0);
-    return (int)q + 1;
+    return (uint32_t)q + 1u;
   }
 };
 

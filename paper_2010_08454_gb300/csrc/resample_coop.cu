@@ -625,10 +625,10 @@ __global__ void __launch_bounds__(kRcTpb, 2) resample_coop_kernel(RcArgs a) {
         // 305, where the runs end in their row or the next).
         const int n_out = (int)(kn - kc);
         const StepDiv dv(u + (uint64_t)kc * stride, stride);
-        int k0 = min(dv.below(base), n_out);
+        int k0 = (int)min(dv.below(base), (uint32_t)n_out);
 #pragma unroll
         for (int r = 0; r < kRcItems; ++r) {
-          const int k1 = min(dv.below(acc_add<FROM_LW>(base, p[r])), n_out);
+          const int k1 = (int)min(dv.below(acc_add<FROM_LW>(base, p[r])), (uint32_t)n_out);
           if (k1 > k0) {
             const int32_t mark = (int32_t)(tid * kRcItems + r) + 1;
             marks[k0] = mark;

@@ -395,11 +395,11 @@ __global__ void __launch_bounds__(kSmcTpb, 1) smc_persistent_kernel(SmcArgs a) {
       const StepDiv dv(offset + (uint64_t)Kb * stride, stride);
       {
         uint64_t c = cstart + texcl;
-        int k0 = min(dv.below(c), n);
+        int k0 = (int)min(dv.below(c), (uint32_t)n);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           c += q[r];
-          const int k1 = min(dv.below(c), n);
+          const int k1 = (int)min(dv.below(c), (uint32_t)n);
           if (k1 > k0) {
             marks[k0] = tid * R + r + 1;
             const int first_row = k0 / 32 + 1, last_row = (k1 - 1) / 32;
@@ -702,9 +702,9 @@ __global__ void __launch_bounds__(kSmcTpb, 1) smc_cluster_kernel(SmcArgs a) {
 #pragma unroll
     for (int r = 0; r < V; ++r) {
       const uint64_t c1 = cstart + inc[r];
-      const int ke = min(dv.below(c1), N);
+      const int ke = (int)min(dv.below(c1), (uint32_t)N);
       int ks = __shfl_up_sync(0xffffffffu, ke, 1);
-      if (lane == 0) ks = min(dv.below(cstart + wbase[r]), N);
+      if (lane == 0) ks = (int)min(dv.below(cstart + wbase[r]), (uint32_t)N);
       auto put = [&](int k, float v) {
         const int to = k / (V * kSmcTpb);
         asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(

@@ -126,3 +126,23 @@ def test_sharded_gather_of_other_records(ppl, words):
                                   state_in=state[b[g]:b[g + 1]].clone()) for g in range(3)]
     assert torch.equal(torch.cat([g[0] for g in got]), anc_ref)
     assert torch.equal(torch.cat([g[1] for g in got]), rec_ref)
+
+
+def test_most_outputs_with_a_stride_of_one(ppl):
+    # the most outputs there are, fixed-point weights whose sum is just below twice
+    # their number: stride 1, and the last chunk's sums lie almost 2^31 positions
+    # past its last output
+    import torch
+    M = (1 << 31) - 1
+    q = torch.ones(2 * 4096, dtype=torch.int64)
+    q[0] = M - 100 - 4095   # chunk 0: the first M - 100 positions
+    q[4096:] = 0
+    q[4096], q[4097], q[5000] = 40, 30, 7
+    q[6000], q[6001] = 100, M - 100 - 30 - 40 - 7 - 100 + 99 + 100
+    total = int(q.sum())
+    assert M <= total < 2 * M
+    anc = ppl.ppl_resample(M, 5, q_fixed=q.cuda())
+    c = torch.cumsum(q.cuda(), 0)
+    for k in range(0, M, 1 << 28):  # output k's position is k: the first sum above it
+        pos = torch.arange(k, min(k + (1 << 28), M), device="cuda")
+        assert torch.equal(anc[k:k + len(pos)].long(), torch.searchsorted(c, pos, right=True))
