@@ -188,13 +188,20 @@ __global__ void __launch_bounds__(kTpb, PPT >= 8 ? 2 : (LEARNED ? 3 : 4)) batche
 // traces and moves when a trace lies kRebaseNats above it; nothing a run
 // computes depends on the other runs, so the result does not depend on timing.
 //
-// 1024 sets x 2^16 traces, 32 points, sorted kernel and this one: 3160 and 2050
-// us under near-posterior proposals, 1700 and 1640 us with prior draws, 1720
-// and 1380 us on 16 points.  A run costs about 13 us of a block besides its
-// traces (the first traces' references, the reduction), so the line lies
-// where runs of 16384 traces fill the blocks several times over; below it
-// prior draws lose (300 x 100000: 755 and 794 us), and above 32 points too,
-// where the padded chains outweigh the sort (64 points: 1055 and 1160 us).
+// Sorted kernel and this one, us, 32 points, near-posterior proposals | prior draws:
+//   256 sets x 2^14 (2^22 traces)   200  173 | 137  141
+//   256 x 2^15 (2^23)               385  329 | 237  267
+//   256 x 2^16 (2^24)               773  547 | 435  446
+//   1024 x 2^14 (2^24)              790  546 | 474  454
+//   1024 x 2^15 (2^25)             1583 1052 | 865  873
+//   1024 x 2^16 (2^26)             3180 2005 | 1654 1657
+// and 1720 and 1380 us for prior draws on 16 points (2^26).  A run costs about 13
+// us of a block besides its traces (the first traces' references, the
+// reduction); smaller batches than these are 2 to 4 times slower here.  Under
+// proposals this kernel wins from 2^22 traces on; prior draws, which skip most
+// traces in either kernel, lose 3 to 13 % up to 2^24 and are even from 2^25 on:
+// the line lies where neither draw loses.  Above 32 points the padded chains
+// outweigh the sort (prior draws, 64 points: 1055 and 1160 us).
 // Both draws take the same kernel, so that a proposal equal to the prior gives
 // the prior's run bit for bit.
 // ---------------------------------------------------------------------------

@@ -392,19 +392,20 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) stats_kernel(
 // HBM bounds it (36 B a particle), if a particle costs few instructions: each
 // lane keeps all four degrees' sums (S, S2 and, per coefficient, sum w d and
 // sum w d^2, d = c - ref) in registers for the whole pass, as f32x2 pairs, and
-// adds a particle to all four with its weight masked by degree: 28 paired
-// multiply-adds and no shuffle, barrier or branch.  The reference (ref, m_ref)
+// adds a particle to all four with its weight masked by degree: 40 paired
+// operations and no shuffle, barrier or branch.  The reference (ref, m_ref)
 // of a degree is shared by the warp's lanes, m_ref within kRebaseNats of the
 // best log-weight the warp has met, so that the weights stay in range and the
 // moments are taken around a point that carries weight.  When a better trace
-// turns up, the lanes move their sums to it exactly (A' = e (A + S g), B' =
-// e (B + g (2 A + S g)), g the shift of the reference, e the ratio of the
+// turns up, the lanes move their sums to it exactly (A' = e A + e S g, B' =
+// e B + g (e A + A'), g the shift of the reference, e the ratio of the
 // weights); a warp's maximum rises about ln(particles) times, so that path is
 // rare.  After 1, 2, 4, .. tiles the reference moves to the warp's weighted
 // mean so far: sums of w d then stay near 0 and round less (around a trace, the
-// mean of 2^22 unit normals came out 1.5 times further off).  Records and log-weights come through a ring of kPostStages cp.async
-// tiles per warp (no register held for a load in flight); nothing is shared
-// between warps until the end.
+// mean of 2^22 unit normals came out 1.5 times further off).  Records and
+// log-weights come through a ring of kPostStages cp.async tiles per warp (no
+// register held for a load in flight); nothing is shared between warps until the
+// end.
 // 2^24 records: 698 us with block-wide tiles of 1024 (56 masked sums reduced by
 // shuffles and ten barriers a tile), 146 us this way (4.1 TB/s; the copy rate would take 89).
 // ---------------------------------------------------------------------------
