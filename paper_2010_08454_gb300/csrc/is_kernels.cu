@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) stats_kernel(
 // register held for a load in flight); nothing is shared between warps until the
 // end.
 // 2^24 records: 698 us with block-wide tiles of 1024 (56 masked sums reduced by
-// shuffles and ten barriers a tile), 146 us this way (4.1 TB/s; the copy rate would take 89).
+// shuffles and ten barriers a tile), 149 us this way (4.1 TB/s; the copy rate would take 89).
 // ---------------------------------------------------------------------------
 constexpr int kPostThreads = 512;  // one block per SM
 constexpr int kPostWarps = kPostThreads / 32;
